@@ -73,7 +73,7 @@ def listed():
                init=0.25, dense_path=2, dense_v_bf16=1),
         # many uneven spectrograms advancing together
         _dense("batch_256_spectrograms_K32", "gamma", 513, 0, 32, 8, 0.0, kind="batch", chains=256, J_lo=200,
-               J_hi=5000, K_true=16, mix="alternate", sweeps=4, dense_path=2),
+               J_hi=5000, K_true=16, mix="alternate", sweeps=2, dense_path=2),
         # one turn of a serving loop: the jobs in flight, each one sweep on
         _dense("batch_serving_12_jobs", "mixed", 0, 0, 0, 8, 0.0, kind="batch", chains=12, J_lo=500,
                J_hi=20000, mix="serving", dense_path=2),
@@ -290,24 +290,27 @@ def work(case):
 _M32 = 0xFFFFFFFF
 
 
-def _normals(seed, t, mat, n, K):
-    """The n x K normals of matrix `mat` at iteration t."""
-    groups = (K + 3) // 4
-    rows = torch.arange(n, device=DEV, dtype=torch.int64)
-    x = [torch.arange(groups, device=DEV, dtype=torch.int64).repeat(n), rows.repeat_interleave(groups),
-         torch.full((n * groups,), t & _M32, device=DEV, dtype=torch.int64),
-         torch.full((n * groups,), ((t >> 32) << 1) | mat, device=DEV, dtype=torch.int64)]
-    k0, k1 = seed & _M32, (seed >> 32) & _M32
+def _normals(t, K, segments):
+    """The n x K normals at iteration t of each segment (seed, matrix, n)."""
+    groups, z = (K + 3) // 4, []
+
+    def per_item(values):
+        return torch.cat([torch.full((n * groups,), v, device=DEV, dtype=torch.int64)
+                          for v, (_, _, n) in zip(values, segments)])
+
+    rows = torch.cat([torch.arange(n, device=DEV) for _, _, n in segments])
+    k0, k1 = (per_item([(seed >> b) & _M32 for seed, _, _ in segments]) for b in (0, 32))
+    x = [torch.arange(groups, device=DEV).repeat(len(rows)), rows.repeat_interleave(groups),
+         torch.full_like(k0, t & _M32), per_item([((t >> 32) << 1) | mat for _, mat, _ in segments])]
     for _ in range(10):
         a, b = x[0] * 0xD2511F53, x[2] * 0xCD9E8D57          # 64-bit products, modulo 2^64
         x = [((b >> 32) & _M32) ^ x[1] ^ k0, b & _M32, ((a >> 32) & _M32) ^ x[3] ^ k1, a & _M32]
         k0, k1 = (k0 + 0x9E3779B9) & _M32, (k1 + 0xBB67AE85) & _M32
     u = [((w >> 9).double() + 0.5) * 2.0 ** -23 for w in x]
-    z = []
     for a, b in ((u[0], u[1]), (u[2], u[3])):
         r = torch.sqrt(-2.0 * torch.log(a))
         z += [r * torch.cos(2 * math.pi * b), r * torch.sin(2 * math.pi * b)]
-    return torch.stack(z, 1).view(n, 4 * groups)[:, :K]
+    return torch.stack(z, 1).view(len(rows), 4 * groups)[:, :K].split([n for _, _, n in segments])
 
 
 def _residual(case, v, mu):
@@ -336,10 +339,14 @@ class _Exact:
         else:
             self.V = _matrix(case, seed)
 
-    def step(self):
+    def segments(self):
+        return [(self.seed, 0, self.case["I"]), (self.seed, 1, self.case["J"])]
+
+    def step(self, normals=None):
         c, self.t = self.case, self.t + 1
-        I, J, K, B = c["I"], c["J"], c["K"], c["B"]
+        I, J, B = c["I"], c["J"], c["B"]
         s, W, H = (self.t - 1) % B, self.W, self.H
+        z = normals or _normals(self.t, c["K"], self.segments())
         GW, GH, n = torch.zeros_like(W), torch.zeros_like(H), 0
         if c["data"] == "ratings":
             n, N = self.first[s + 1] - self.first[s], len(self.v)
@@ -362,9 +369,9 @@ class _Exact:
         eps = (c["eps_a"] / self.t) ** c["eps_b"] if "eps_a" in c else c["eps"]
         S = N / n if n else 0.0
         out = []
-        for mat, (x, g) in enumerate(((W, GW), (H, GH))):
-            prior = -torch.ones_like(x) if c["prior"] == EXPON else -x
-            y = x + eps * (S * g + prior) + math.sqrt(2 * eps) * _normals(self.seed, self.t, mat, len(x), K)
+        for x, g, zx in ((W, GW, z[0]), (H, GH, z[1])):
+            prior = -1.0 if c["prior"] == EXPON else -x
+            y = x + eps * (S * g + prior) + math.sqrt(2 * eps) * zx
             out.append(y.abs() if c["prior"] == EXPON else y)
         self.W, self.H = out
 
@@ -403,13 +410,14 @@ def exact(case, seed):
             out += [m, s2 / n - m * m]
         return (*out, int(n))
     if kind == "batch":
-        out = []
-        for k, m in enumerate(_members(case)):
-            x = _Exact(m, seed + 17 * k)
-            for _ in range(m["sweeps"] * m["B"]):
-                x.step()
-            out += [x.W.reshape(-1), x.H.reshape(-1)]
-        return torch.cat(out)
+        chains = [_Exact(m, seed + 17 * k) for k, m in enumerate(_members(case))]
+        for t in range(1, case["sweeps"] * case["B"] + 1):
+            for K in sorted({x.case["K"] for x in chains}):      # one K's normals together
+                mine = [x for x in chains if x.case["K"] == K]
+                z = _normals(t, K, [q for x in mine for q in x.segments()])
+                for k, x in enumerate(mine):
+                    x.step(z[2 * k:2 * k + 2])
+        return torch.cat([f.reshape(-1) for x in chains for f in (x.W, x.H)])
     x = _Exact(case, seed)
     if kind == "evaluate":
         return _evaluate(x, 25)
