@@ -528,7 +528,7 @@ def run_ours(args, wl_name, wl):
         share = grad_ms / max(kern_ms, 1e-12)
         roofline = {"bound": "hbm", "achieved": achieved, "peak": hbm_peak, "unit": "GB/s",
                     "frac": achieved / hbm_peak, "traffic": kernel_traffic(wl_name),
-                    "kernel": "part_step (gradient kernel + update kernel)", "kernel_ms": part_ms,
+                    "kernel": "part_step (gradient and update)", "kernel_ms": part_ms,
                     "kernel_ms_source": "timed sweeps / B",
                     "grad_share": share, "update_share": 1.0 - share,
                     "profiled_grad_kernel_ms": grad_ms, "profiled_update_kernel_ms": upd_ms,
@@ -551,9 +551,9 @@ def run_ours(args, wl_name, wl):
         "roofline": roofline,
         # per sweep: B x (gradient + update) + 2 accumulate + advance t + set t
         # per part-step: the chain kernel and the update (tensor-core path),
-        # or each side's gradient and update on two streams (sparse path);
-        # per sweep four more (posterior sums of W and H, the t counter)
-        "gpu_launches": args.steps * ((2 if tensor_path(wl) else 4) * wl["B"] + 4),
+        # or one launch of both (sparse path); per sweep one more (posterior
+        # sums and the t counter)
+        "gpu_launches": args.steps * ((2 if tensor_path(wl) else 1) * wl["B"] + 1),
         "clocks": clocks,
         "rmse_after": rmse,
     }
@@ -1229,9 +1229,9 @@ def run_serving(args, wl_name, wl):
         "peak_budget_used_bytes": st["peak_bytes"],
         "roofline": None,
         # per batch sweep: set t, B x (gradient launches per kernel variant
-        # (about two) + update), accumulate, advance t; standing chain: 2B + 3
+        # (about two) + update), accumulate, advance t; standing chain: 2B + 1
         # per sweep
-        "gpu_launches": st["sweeps"] * (3 * wl["B"] + 3) + r["st_sweeps"] * (2 * 16 + 3),
+        "gpu_launches": st["sweeps"] * (3 * wl["B"] + 3) + r["st_sweeps"] * (2 * 16 + 1),
         "clocks": r["clocks"],
         "e2e": {"value": value, "unit": UNIT, "h2d_bytes_per_step": h2d / max(1, len(jobs)),
                 "d2h_bytes_per_step": d2h / max(1, len(jobs)),

@@ -117,11 +117,11 @@ typedef struct {
                                * stay BF16.  Needs dense_path 1 or 3, K <= 128,
                                * FP32 V (dense_path 1 then always takes the
                                * single-pass kernel). */
-    int32_t gather_bf16;      /* 1: on the sparse path the gradient kernel gathers
-                               * BF16 copies of the other factor's rows (half the
-                               * bytes; the own row, the products and all sums stay
-                               * FP32); the copies are rebuilt by psgld_set_factors
-                               * and rewritten by every update.  Set it before
+    int32_t gather_bf16;      /* 1: on the sparse path the part-step gathers BF16
+                               * copies of the other factor's rows (half the bytes;
+                               * the own row, the products and all sums stay FP32);
+                               * the copies are rebuilt by psgld_set_factors and
+                               * written by every part-step.  Set it before
                                * psgld_set_factors. */
     int32_t max_sms;          /* > 0: the two-sided tensor-core kernel (persistent,
                                * one CTA per SM) runs on at most this many SMs, so
@@ -140,14 +140,15 @@ typedef struct {
                                * not depend on it. */
     int32_t debug_wait_polls; /* for testing the timeout path; 0 (the default): the
                                * normal limit of every bounded device wait (2^24
-                               * polls or about one second of SM clock).  > 0: the
-                               * sparse gradient kernel's first wait for its row
-                               * gathers makes at most this many polls, without
-                               * suspending and before it issues the copies, then
-                               * gives up -- a wait that surely runs out, on
-                               * purpose: the kernel sets the context's error
-                               * flag, waits for its own copies with the normal
-                               * limit, and the next synchronising call returns
+                               * polls or about one second of SM clock).  > 0: each
+                               * block of the sparse part-step kernel first makes
+                               * a bulk copy of a row and waits for it with at
+                               * most this many polls, made before it issues the
+                               * copy -- a wait that surely runs out, on purpose:
+                               * the kernel sets the context's error flag, waits
+                               * for the copy with the normal limit and returns
+                               * without a step, and the next synchronising call
+                               * returns
                                * PSGLD_ERR_TIMEOUT naming the kernel and the wait.
                                * The part-step's result is then undefined; the
                                * context stays usable (set the factors again). */
@@ -351,9 +352,10 @@ PSGLD_API psgld_status psgld_part_layout(psgld_ctx *ctx, int32_t s, int32_t *row
  * the context's last stream. */
 PSGLD_API psgld_status psgld_profile_read(psgld_ctx *ctx, double *total_ms_host,
                                           int64_t *launches_host);
-/* The same split at the end of the gradient kernel (the sparse gather kernel
- * or the tensor-core chain): *grad_ms_host and *update_ms_host receive the
- * summed durations of the gradient and of the update launches. */
+/* The same split at the end of the tensor-core chain: *grad_ms_host and
+ * *update_ms_host receive the summed durations of the gradient and of the
+ * update launches.  On the sparse path gradient and update are one launch,
+ * counted as the gradient's. */
 PSGLD_API psgld_status psgld_profile_read_split(psgld_ctx *ctx, double *grad_ms_host,
                                                 double *update_ms_host, int64_t *launches_host);
 

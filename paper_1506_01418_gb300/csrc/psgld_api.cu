@@ -224,7 +224,7 @@ bool ready(psgld_ctx *c, psgld_status *s)
 {
     if (!c->has_data) { *s = fail(c, PSGLD_ERR_STATE, "no data set"); return false; }
     if (!c->has_factors) { *s = fail(c, PSGLD_ERR_STATE, "no factors set"); return false; }
-    if (c->opt.gather_bf16 && !c->dense && !(c->W16 && c->H16)) {
+    if (c->opt.gather_bf16 && !c->dense && !gather_bf16(c)) {
         *s = fail(c, PSGLD_ERR_STATE, "gather_bf16 was enabled after the factors were set: set them again");
         return false;
     }
@@ -237,11 +237,10 @@ psgld_status capture_sweep(psgld_ctx *c, bool acc, cudaGraphExec_t *out)
     cudaStream_t cs = c->capture_stream;
     const int w0 = c->wcur, h0 = c->hcur;
     PSGLD_CK(c, cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
-    psgld_status s = PSGLD_OK;
+    psgld_status s = c->opt.eps_mode == PSGLD_EPS_POLY ? launch_eps_table(c, cs) : PSGLD_OK;
     for (int b = 0; b < c->B && s == PSGLD_OK; ++b)
         s = launch_part_step(c, b + 1, c->t_dev, b + 1, cs);
-    if (s == PSGLD_OK && acc) s = launch_accumulate(c, cs);
-    if (s == PSGLD_OK) s = launch_advance_t(c, c->B, cs);
+    if (s == PSGLD_OK) s = launch_finish_sweep(c, acc, c->B, cs);
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaStreamEndCapture(cs, &g);
     c->wcur = w0;
@@ -334,10 +333,6 @@ psgld_status create_context(int64_t I, int64_t J, int32_t K, int32_t B, double t
     // after the legacy stream)
     if (cudaStreamCreateWithFlags(&c->capture_stream, cudaStreamNonBlocking) != cudaSuccess)
         s = fail(c, PSGLD_ERR_CUDA, "stream creation failed");
-    if (s == PSGLD_OK && (cudaStreamCreateWithFlags(&c->side_stream, cudaStreamNonBlocking) != cudaSuccess ||
-                          cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
-                          cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming) != cudaSuccess))
-        s = fail(c, PSGLD_ERR_CUDA, "stream or event creation failed");
     cudaStream_t zs = c->capture_stream;
     for (int b = 0; b < 2 && s == PSGLD_OK; ++b) {
         s = alloc(c, &c->W[b], I * c->ldk, true, zs);
@@ -351,8 +346,8 @@ psgld_status create_context(int64_t I, int64_t J, int32_t K, int32_t B, double t
     if (s == PSGLD_OK) s = alloc(c, &c->red, reduce_blocks(), true, zs);
     if (s == PSGLD_OK) s = alloc(c, &c->flag, 1, true, zs);
     if (s == PSGLD_OK) s = alloc(c, &c->kflag, 1, true, zs);
-    if (s == PSGLD_OK) s = prepare_kernels(c);
     if (s == PSGLD_OK) s = alloc(c, &c->t_dev, 1, true, zs);
+    if (s == PSGLD_OK) s = alloc(c, &c->eps_tab, B, true, zs);
     if (s == PSGLD_OK) c->red_host.assign(reduce_blocks(), 0.0);
     if (s == PSGLD_OK && cudaStreamSynchronize(zs) != cudaSuccess)
         s = fail(c, PSGLD_ERR_CUDA, "zero fill failed");
@@ -636,8 +631,11 @@ psgld_status psgld_sweep(psgld_ctx *c, int32_t n_sweeps, void *stream)
     if (n_sweeps == 0) return PSGLD_OK;
     const bool graphs = c->opt.use_graphs && c->opt.part_mode == 0;
     if (graphs) {
-        set_t_kernel<<<1, 32, 0, st>>>(c->t_dev, c->t_done);
-        PSGLD_CK(c, cudaGetLastError());
+        if (c->t_dev_is != c->t_done) {   // part-steps launched directly leave the counter behind
+            set_t_kernel<<<1, 32, 0, st>>>(c->t_dev, c->t_done);
+            PSGLD_CK(c, cudaGetLastError());
+        }
+        c->t_dev_is = -1;                 // until every replay is enqueued
     }
     for (int32_t n = 0; n < n_sweeps; ++n) {
         const bool acc = c->sweeps_done >= c->opt.burn_in_sweeps;
@@ -659,7 +657,7 @@ psgld_status psgld_sweep(psgld_ctx *c, int32_t n_sweeps, void *stream)
                 if (s != PSGLD_OK) return s;
             }
             if (acc) {
-                s = launch_accumulate(c, st);
+                s = launch_finish_sweep(c, true, 0, st);
                 if (s != PSGLD_OK) return s;
             }
         }
@@ -667,6 +665,7 @@ psgld_status psgld_sweep(psgld_ctx *c, int32_t n_sweeps, void *stream)
         c->sweeps_done += 1;
         if (acc) c->n_samples += 1;
     }
+    if (graphs) c->t_dev_is = c->t_done;
     mark_enqueued(c, st);
     return PSGLD_OK;
 }
@@ -741,7 +740,7 @@ psgld_status psgld_set_state(psgld_ctx *c, const double *sW, const double *sW2, 
     // the padding columns (K .. ldk-1) stay as they are: zero
     for (const auto &q : parts)
         PSGLD_CK(c, cudaMemcpy2D(q.dst, pitch, q.src, row, row, (size_t)q.rows, cudaMemcpyHostToDevice));
-    PSGLD_CK(c, cudaMemcpy(c->t_dev, &t, sizeof t, cudaMemcpyHostToDevice));
+    c->t_dev_is = -1;
     c->t_done = t;
     c->sweeps_done = sweeps;
     c->n_samples = samples;
@@ -1053,6 +1052,7 @@ psgld_status psgld_batch_sweep(psgld_ctx *const *ctxs, int32_t n, int32_t n_swee
             }
             c->t_done += (int64_t)B * n_sweeps;
         }
+        c->t_dev_is = s == PSGLD_OK ? c->t_done : -1;
         // after a failed launch the factors are unspecified (set them again),
         // but whatever was enqueued is still waited for before the context
         // frees its memory
@@ -1082,11 +1082,12 @@ int64_t psgld_estimate_device_bytes(int64_t I, int64_t J, int32_t K, int32_t B, 
     // psgld_create: W, Ht (two buffers each), G, FP64 posterior sums, reduction slots
     bytes += 2 * (I + J) * ldk * 4 + (I + J) * ldk * 4 + 2 * (I + J) * ldk * 8 + reduce_blocks() * 8 + 64;
     if (dense_path == 0) {
-        // the two part-major entry layouts and their partial-sum slots
-        const int unit = unit_entries((K + 3) / 4);
+        // the two part-major entry layouts, the A side's row of each entry,
+        // the lists of the rows with many entries and their chunks' sums
         for (int side = 0; side < 2; ++side) {
             const int64_t n_rows = side == 0 ? I : J;
-            bytes += (B * n_rows + 1) * 4 + nnz * 12 + 2 * (cdiv(nnz, unit) + B) * ldk * 4;
+            bytes += (B * n_rows + 1) * 4 + nnz * (side == 0 ? 12 : 8) + 4 * std::min(nnz / (light_row_for(I + J) + 1), B * n_rows) +
+                     8 * max_chunks(nnz) + (4 * ldk + 4) * std::min(max_chunks(nnz), max_chunks(cdiv(nnz, B)) + n_rows);
         }
         return bytes;
     }
@@ -1128,18 +1129,16 @@ void psgld_destroy(psgld_ctx *c)
         cudaEventDestroy(c->bdone);
     }
     dev_free(c, c->bscratch);
-    dev_free(c, c->W16);
-    dev_free(c, c->H16);
-    for (int b = 0; b < 2; ++b) { dev_free(c, c->W[b]); dev_free(c, c->Ht[b]); }
+    for (int b = 0; b < 2; ++b) {
+        dev_free(c, c->W[b]);
+        dev_free(c, c->Ht[b]);
+        dev_free(c, c->W16[b]);
+        dev_free(c, c->H16[b]);
+    }
     dev_free(c, c->G);
     dev_free(c, c->sW.s); dev_free(c, c->sW.s2); dev_free(c, c->sH.s); dev_free(c, c->sH.s2);
     dev_free(c, c->red); dev_free(c, c->flag); dev_free(c, c->kflag); dev_free(c, c->t_dev);
-    if (c->side_stream) {
-        cudaStreamSynchronize(c->side_stream);
-        cudaStreamDestroy(c->side_stream);
-    }
-    if (c->ev_fork) cudaEventDestroy(c->ev_fork);
-    if (c->ev_join) cudaEventDestroy(c->ev_join);
+    dev_free(c, c->eps_tab);
     if (c->capture_stream) cudaStreamDestroy(c->capture_stream);
     delete c;
 }

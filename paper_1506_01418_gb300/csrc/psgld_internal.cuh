@@ -4,14 +4,13 @@
 //   W[2]  : I x ldk fp32, row-major, ping-pong pair (ldk = 4*ceil(K/4); the
 //           padding columns are kept at zero so every row is float4-aligned)
 //   Ht[2] : J x ldk fp32, H transposed, same rules
-//   G     : (I + J) x ldk fp32, the likelihood gradient of the current
-//           part-step (rows 0..I-1 for W, I..I+J-1 for H^T)
+//   G     : (I + J) x ldk fp32, dense path: the likelihood gradient of the
+//           current part-step (rows 0..I-1 for W, I..I+J-1 for H^T)
 //   A-side layout (part-major CSR): entries ordered by (part s, row i, col j)
 //           ptrA[s*I + i] .. ptrA[s*I + i + 1] -> idxA (col j), valA (v)
 //   B-side layout (part-major CSC): entries ordered by (part s, col j, row i)
 //           ptrB[s*J + j] .. -> idxB (row i), valB (v)
-//   segA/segB : per part, the chunk records of the fused part-step kernel:
-//           one per (heavy row, run of at most chunk_len entries)
+//   mid/heavy, per side: per part, the rows with many entries in it
 //   posterior sums: fp64 copies of W, W^2, Ht, Ht^2 (padded like the factors)
 //   dense tensor-core path instead of the two layouts:
 //   Vd    : I x J fp32, row-major (ldv = J)
@@ -22,8 +21,8 @@
 //           swizzled MMA tiles per piece (dev::shadow_store4); Et, one part's
 //           E in 128 x 64 BF16 tiles (written by the rows items, read by the
 //           columns items); tsync, the kernel's claim and block counters
-//   sparse path with gather_bf16: W16 / H16, BF16 copies of W and H^T, rows
-//           of ldk rounded up to 8, rewritten by every update
+//   sparse path with gather_bf16: W16[2] / H16[2], BF16 copies of W and H^T,
+//           rows of ldk rounded up to 8, written by every part-step
 #pragma once
 
 #include <cuda_bf16.h>
@@ -43,12 +42,25 @@ struct SideLayout {
     int32_t *ptr = nullptr;    // B*n_rows + 1 entry offsets (absolute)
     int32_t *idx = nullptr;    // other index of each entry
     float *val = nullptr;      // value of each entry
-    int32_t *own = nullptr;    // own row of each entry
-    std::vector<int64_t> part_first;   // B+1: first entry of each part
-    int64_t max_units = 0;     // most units (unit_entries consecutive entries) in one part
-    float *partial = nullptr;  // 2 x max_units x ldk: head / tail partial
-                               // sums of rows that cross a unit boundary
+    int32_t *own = nullptr;    // A side: own row of each entry (log-likelihood, RMSE)
+    // per part, the rows with more than light_row and at most kMidRow entries
+    // in it, ascending, and the chunks (row, number) of kChunk entries of the
+    // rows with more; part s: [first[s], first[s + 1])
+    int32_t *mid = nullptr;
+    int2 *heavy = nullptr;
+    std::vector<int64_t> mid_first, heavy_first;
+    float *partial = nullptr;  // ldk sums per chunk of the part with the most chunks
+    int *arrived = nullptr;    // per chunk: of a row's first one, how many are done
 };
+
+// Entries of a row in one part up to which a warp takes the row
+// (psgld_rows.cu); above, a block takes each kChunk.
+constexpr uint32_t kMidRow = 128, kChunk = 512;
+// ... and up to which one of a warp's teams of lanes does: few when the rows
+// of a part do not fill the chip's warps anyway.
+constexpr int light_row_for(int64_t rows) { return rows < 152 * 32 ? 2 : 16; }
+// chunks of rows with more than kMidRow entries, at most, among n entries
+constexpr int64_t max_chunks(int64_t n) { return n / kChunk + n / kMidRow; }
 
 struct Sums {
     double *s = nullptr, *s2 = nullptr;
@@ -94,7 +106,8 @@ struct psgld_ctx {
     uint16_t *Et = nullptr;                     // E tiles of one part (BF16)
     int *tsync = nullptr;                       // two-sided kernel counters: 2 + B ints
     uint16_t *Wsh = nullptr, *Hsh = nullptr;    // BF16 shadows of W, H^T
-    uint16_t *W16 = nullptr, *H16 = nullptr;    // sparse path, gather_bf16: BF16 copies of W, H^T
+    // sparse path, gather_bf16: BF16 copies of both buffers of W and H^T
+    uint16_t *W16[2] = {nullptr, nullptr}, *H16[2] = {nullptr, nullptr};
     int mt_max = 0, nt_max = 0;      // 128-row tiles per row piece / column piece
     int nt2_max = 0;                 // 256-row column tiles per column piece (columns items)
     int ni_max = 0, nj_max = 0;      // 64-row tiles per row piece / column piece
@@ -131,10 +144,9 @@ struct psgld_ctx {
     cudaGraphExec_t graph_acc[4] = {nullptr, nullptr, nullptr, nullptr};
     cudaStream_t capture_stream = nullptr;
     int64_t *t_dev = nullptr;    // iteration counter read by graph replays
-    // sparse part-steps: the rows of H^T on a second stream, forked from and
-    // joined back into the launch stream
-    cudaStream_t side_stream = nullptr;
-    cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+    int light_row = 0;           // most entries in a part of a row that one team takes (psgld_rows.cu)
+    int64_t t_dev_is = -1;       // its value after the work enqueued so far (-1: unknown)
+    float2 *eps_tab = nullptr;   // captured sweeps with eps_t: (eps, sqrt(2 eps)) of each part-step
     psgld::BatchGraphs bgraphs;  // captured batch sweeps while this context leads a batch
 
     // psgld_batch_sweep's parameter tables while this context leads a batch
@@ -190,20 +202,19 @@ int part_of_iteration(const psgld_ctx *c, int64_t t);
 // Enqueue iteration t.  When t_dev is non-null the kernels read t from
 // *t_dev + t_add instead (used inside captured graphs); `t` then only
 // selects the part and must satisfy (t-1) % B == part.
-// Sparse path with gather_bf16: the gradient kernel gathers BF16 copies of
-// the factors (rows of ldk rounded up to 8), kept by the update kernel and
-// built from the current factors by build_gather_shadows (allocating them).
-bool gather_bf16(const psgld_ctx *c);
-psgld_status build_gather_shadows(psgld_ctx *c, cudaStream_t st);
-
 psgld_status launch_part_step(psgld_ctx *c, int64_t t, const int64_t *t_dev,
                               int64_t t_add, cudaStream_t st);
 
-// One-time kernel attributes (dynamic shared memory) for this context's K.
-psgld_status prepare_kernels(psgld_ctx *c);
-// Entries per work unit of the gradient kernel for a factor width of
-// ngroups float4 groups.
-int unit_entries(int ngroups);
+// ---- sparse part-step (psgld_rows.cu) ----------------------------------------
+// The one launch of part `part` at iteration t (or *t_dev + t_add); does not
+// flip the context's buffers.
+psgld_status launch_rows(psgld_ctx *c, int part, int64_t t, const int64_t *t_dev, int64_t t_add, cudaStream_t st);
+// With gather_bf16 the part-step gathers BF16 copies of the factors (rows of
+// ldk rounded up to 8) and writes those of the new ones; built from the
+// current factors by build_gather_shadows (allocating them).
+bool gather_bf16(const psgld_ctx *c);
+psgld_status build_gather_shadows(psgld_ctx *c, cudaStream_t st);
+
 // After a synchronisation point: PSGLD_ERR_TIMEOUT (and the flag cleared) if
 // a sampling kernel reported a bounded wait that ran out, else PSGLD_OK.
 psgld_status check_kernel_flag(psgld_ctx *c);
@@ -260,8 +271,11 @@ psgld_status launch_accumulate_batch(psgld_ctx *c0, const void *params, const in
 psgld_status launch_t_batch(psgld_ctx *c0, const void *params, int n, int mode, cudaStream_t st);
 
 // ---- reductions (psgld_reduce.cu) -----------------------------------------
-psgld_status launch_accumulate(psgld_ctx *c, cudaStream_t st);
-psgld_status launch_advance_t(psgld_ctx *c, int64_t by, cudaStream_t st);
+// Both factors added to the posterior sums (acc), the device counter t
+// advanced by `by` (by > 0), in one launch.
+psgld_status launch_finish_sweep(psgld_ctx *c, bool acc, int64_t by, cudaStream_t st);
+// eps_tab[b] for the part-steps t = *t_dev + b + 1 of a captured sweep.
+psgld_status launch_eps_table(psgld_ctx *c, cudaStream_t st);
 psgld_status reduce_loglik_rmse(psgld_ctx *c, int mode, int use_mean,
                                 cudaStream_t st, double *out);
 

@@ -10,9 +10,9 @@
 // Both are produced by a stable LSD radix sort written here (8-bit digits,
 // per-tile histograms, a global exclusive scan and a stable scatter whose
 // in-tile ranks come from warp match/ballot), so the order is exact and
-// repeatable.  Every entry also records its own row (the row of W for the
-// A side, the row of H^T for the B side), so that the part-step kernel can
-// take any 32 consecutive entries of a part as one unit of work.
+// repeatable.  The A side's entries also record their row of W, for the
+// reductions over all entries, and both sides list, per part, the rows with
+// many entries, which the part-step gives more lanes.
 #include <algorithm>
 
 #include "psgld_internal.cuh"
@@ -252,17 +252,42 @@ __global__ void finish_side(int64_t nnz, const uint64_t *__restrict__ key,
             const uint32_t e = perm[p];
             idx[p] = other[e];
             val[p] = vv[e];
-            own[p] = (int32_t)(slot % n_rows);
+            if (own) own[p] = (int32_t)(slot % n_rows);
             if (p > 0 && key[p] == key[p - 1]) atomicOr(flag, 4);
         }
     }
 }
 
-__global__ void gather_ptr(const int32_t *__restrict__ ptr, int64_t n_rows, int B,
-                           int64_t *__restrict__ out)
+// Per slot (row of a part): is it a mid row (heavy = 0), or how many chunks
+// has it as a heavy one
+__global__ void count_rows(const int32_t *__restrict__ ptr, int64_t nslots, int heavy, uint32_t light,
+                           uint32_t *__restrict__ out)
 {
-    const int s = threadIdx.x;
-    if (s <= B) out[s] = ptr[(int64_t)s * n_rows];
+    for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < nslots;
+         s += (int64_t)gridDim.x * blockDim.x) {
+        const uint32_t n = (uint32_t)(ptr[s + 1] - ptr[s]);
+        out[s] = heavy ? (n > kMidRow ? (n + kChunk - 1) / kChunk : 0u) : (n > light && n <= kMidRow ? 1u : 0u);
+    }
+}
+
+// The mid rows, or the heavy rows' chunks, in slot order (pos: exclusive
+// scan of count_rows).
+__global__ void list_rows(const uint32_t *__restrict__ pos, int64_t nslots, int64_t n_rows,
+                          int32_t *__restrict__ mid, int2 *__restrict__ heavy)
+{
+    for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < nslots;
+         s += (int64_t)gridDim.x * blockDim.x) {
+        const uint32_t a = pos[s], b = pos[s + 1];
+        if (mid && b > a) mid[a] = (int32_t)(s % n_rows);
+        if (heavy)
+            for (uint32_t k = a; k < b; ++k) heavy[k] = make_int2((int)(s % n_rows), (int)(k - a));
+    }
+}
+
+// out[s] = x[s n_rows], s = 0 .. B: where each part begins
+__global__ void gather_starts(const uint32_t *__restrict__ x, int64_t n_rows, int B, int64_t *__restrict__ out)
+{
+    for (int s = threadIdx.x; s <= B; s += blockDim.x) out[s] = x[(int64_t)s * n_rows];
 }
 
 int grid_for(int64_t n, int threads)
@@ -323,7 +348,8 @@ void free_layout(psgld_ctx *c)
     if (c->capture_stream) cudaStreamSynchronize(c->capture_stream);
     for (auto &sd : c->side) {
         dev_free(c, sd.ptr); dev_free(c, sd.idx); dev_free(c, sd.val); dev_free(c, sd.own);
-        dev_free(c, sd.partial);
+        dev_free(c, sd.mid); dev_free(c, sd.heavy);
+        dev_free(c, sd.partial); dev_free(c, sd.arrived);
         sd = SideLayout{};
     }
     dev_free(c, c->Vd);
@@ -360,6 +386,7 @@ psgld_status build_layout(psgld_ctx *c, int64_t nnz, const int32_t *i_dev, const
     const int bitsA = bits_for((uint64_t)(B * I)) + bitsJ;
     const int bitsB = bits_for((uint64_t)(B * J)) + bitsI;
     const int64_t n = nnz;
+    c->light_row = light_row_for(I + J);
 
     uint64_t *kA = nullptr, *kB = nullptr, *kt = nullptr;
     uint32_t *pA = nullptr, *pB = nullptr, *pt = nullptr;
@@ -384,7 +411,7 @@ psgld_status build_layout(psgld_ctx *c, int64_t nnz, const int32_t *i_dev, const
     PSGLD_ALLOC(pA, n); PSGLD_ALLOC(pB, n); PSGLD_ALLOC(pt, n);
     PSGLD_ALLOC(hist, scan_n); PSGLD_ALLOC(hscan, scan_n + 1); PSGLD_ALLOC(tmp, tmp_n);
     int64_t *offs_dev = nullptr;
-    PSGLD_ALLOC(offs_dev, B + 1);
+    PSGLD_ALLOC(offs_dev, 3 * ((int64_t)B + 1));   // starts of the parts' entries, mid and heavy rows
 #undef PSGLD_ALLOC
 
     auto ck = [&](cudaError_t e, const char *what) -> psgld_status {
@@ -418,27 +445,42 @@ psgld_status build_layout(psgld_ctx *c, int64_t nnz, const int32_t *i_dev, const
         s = dmalloc(c, &sd.ptr, nslots + 1);
         if (s == PSGLD_OK) s = dmalloc(c, &sd.idx, n);
         if (s == PSGLD_OK) s = dmalloc(c, &sd.val, n);
-        if (s == PSGLD_OK) s = dmalloc(c, &sd.own, n);
+        if (s == PSGLD_OK && side == 0) s = dmalloc(c, &sd.own, n);
+        if (s == PSGLD_OK) s = dmalloc(c, &sd.mid, std::min(n / (c->light_row + 1), nslots));
+        if (s == PSGLD_OK) s = dmalloc(c, &sd.heavy, max_chunks(n));
         if (s != PSGLD_OK) { cleanup(); free_layout(c); return s; }
         finish_side<<<grid_for(n + 1, 256), 256, 0, st>>>(n, k0, v0, side == 0 ? j_dev : i_dev, v_dev,
                                                           side == 0 ? bitsJ : bitsI, nslots, n_rows,
                                                           sd.idx, sd.val, sd.own, sd.ptr, c->flag);
         if ((s = ck(cudaGetLastError(), "finish_side")) != PSGLD_OK) return s;
-        gather_ptr<<<1, 128, 0, st>>>(sd.ptr, n_rows, B, offs_dev);
-        std::vector<int64_t> h(B + 1);
+        gather_starts<<<1, 128, 0, st>>>(reinterpret_cast<const uint32_t *>(sd.ptr), n_rows, B, offs_dev);
+        for (int k = 0; k < 2; ++k) {
+            count_rows<<<grid_for(nslots, 256), 256, 0, st>>>(sd.ptr, nslots, k, (uint32_t)c->light_row, hist);
+            s = exclusive_scan(c, hist, hscan, nslots, tmp, st);
+            if (s != PSGLD_OK) { cleanup(); free_layout(c); return s; }
+            list_rows<<<grid_for(nslots, 256), 256, 0, st>>>(hscan, nslots, n_rows, k == 0 ? sd.mid : nullptr,
+                                                             k == 0 ? nullptr : sd.heavy);
+            gather_starts<<<1, 128, 0, st>>>(hscan, n_rows, B, offs_dev + (k + 1) * (B + 1));
+        }
+        if ((s = ck(cudaGetLastError(), "row lists")) != PSGLD_OK) return s;
+        std::vector<int64_t> h(3 * (size_t)(B + 1));
         if ((s = ck(cudaMemcpyAsync(h.data(), offs_dev, sizeof(int64_t) * h.size(), cudaMemcpyDeviceToHost, st), "offsets d2h")) != PSGLD_OK) return s;
         if ((s = ck(cudaStreamSynchronize(st), "sync")) != PSGLD_OK) return s;
-        sd.part_first = h;
         if (side == 0) {
             c->part_n.resize(B);
             for (int p = 0; p < B; ++p) c->part_n[p] = h[p + 1] - h[p];
         }
-        const int unit = unit_entries(c->ngroups);
-        sd.max_units = 0;
-        for (int p = 0; p < B; ++p)
-            sd.max_units = std::max<int64_t>(sd.max_units, (h[p + 1] - h[p] + unit - 1) / unit);
-        s = dmalloc(c, &sd.partial, 2 * std::max<int64_t>(1, sd.max_units) * c->ldk);
-        if (s != PSGLD_OK) { cleanup(); free_layout(c); return s; }
+        sd.mid_first.assign(h.begin() + (B + 1), h.begin() + 2 * (B + 1));
+        sd.heavy_first.assign(h.begin() + 2 * (B + 1), h.end());
+        int64_t chunks = 0;
+        for (int p = 0; p < B; ++p) chunks = std::max(chunks, sd.heavy_first[p + 1] - sd.heavy_first[p]);
+        if (chunks > 0) {
+            s = dmalloc(c, &sd.partial, chunks * c->ldk);
+            if (s == PSGLD_OK) s = dmalloc(c, &sd.arrived, chunks);
+            if (s != PSGLD_OK) { cleanup(); free_layout(c); return s; }
+            if ((s = ck(cudaMemsetAsync(sd.arrived, 0, sizeof(int) * (size_t)chunks, st), "memset chunks")) != PSGLD_OK)
+                return s;
+        }
     }
     if ((s = ck(cudaMemcpyAsync(&hflag, c->flag, sizeof(int), cudaMemcpyDeviceToHost, st), "flag d2h")) != PSGLD_OK) return s;
     if ((s = ck(cudaStreamSynchronize(st), "sync")) != PSGLD_OK) return s;

@@ -18,19 +18,45 @@
 namespace psgld {
 namespace {
 
-__global__ void accumulate_kernel(const float4 *__restrict__ x, int64_t n4, double *__restrict__ s,
-                                  double *__restrict__ s2)
+__device__ __forceinline__ void accumulate4(const float4 v, double2 *ps, double2 *ps2)
 {
-    for (int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; a < n4;
+    double2 p0 = ps[0], p1 = ps[1], q0 = ps2[0], q1 = ps2[1];
+    const double a0 = v.x, a1 = v.y, a2 = v.z, a3 = v.w;
+    p0.x += a0; p0.y += a1; p1.x += a2; p1.y += a3;
+    q0.x += a0 * a0; q0.y += a1 * a1; q1.x += a2 * a2; q1.y += a3 * a3;
+    ps[0] = p0; ps[1] = p1; ps2[0] = q0; ps2[1] = q1;
+}
+
+// The end of a sweep: both factors' float4 groups (W first) added to their
+// sums, and the iteration counter advanced, in one launch (a small chain's
+// sweep is bound by its launches).
+struct FinishParams {
+    const float4 *x[2];
+    double *s[2], *s2[2];
+    int64_t n0, n;            // groups of W, of both (0: nothing to add)
+    int64_t *t;               // or null
+    int64_t by;
+};
+
+__global__ void finish_sweep_kernel(const __grid_constant__ FinishParams P)
+{
+    if (P.t && blockIdx.x == 0 && threadIdx.x == 0) *P.t += P.by;
+    for (int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; a < P.n;
          a += (int64_t)gridDim.x * blockDim.x) {
-        const float4 v = x[a];
-        double2 *ps = reinterpret_cast<double2 *>(s) + 2 * a;
-        double2 *ps2 = reinterpret_cast<double2 *>(s2) + 2 * a;
-        double2 p0 = ps[0], p1 = ps[1], q0 = ps2[0], q1 = ps2[1];
-        const double a0 = v.x, a1 = v.y, a2 = v.z, a3 = v.w;
-        p0.x += a0; p0.y += a1; p1.x += a2; p1.y += a3;
-        q0.x += a0 * a0; q0.y += a1 * a1; q1.x += a2 * a2; q1.y += a3 * a3;
-        ps[0] = p0; ps[1] = p1; ps2[0] = q0; ps2[1] = q1;
+        const int f = a >= P.n0;
+        const int64_t u = f ? a - P.n0 : a;
+        accumulate4(P.x[f][u], reinterpret_cast<double2 *>(P.s[f]) + 2 * u,
+                    reinterpret_cast<double2 *>(P.s2[f]) + 2 * u);
+    }
+}
+
+// eps_t = (a / t)^b and sqrt(2 eps_t) of the B part-steps after *t: FP64
+// power functions, once per part-step instead of once per thread of it.
+__global__ void eps_table_kernel(const int64_t *t, int B, double a, double b, float2 *out)
+{
+    for (int k = threadIdx.x; k < B; k += blockDim.x) {
+        const double e = pow(a / (double)(*t + k + 1), b);
+        out[k] = make_float2((float)e, (float)sqrt(2.0 * e));
     }
 }
 
@@ -48,7 +74,7 @@ struct AccParams {
 
 // Every context's factors added to its sums in one launch: context i owns
 // float4 units [unit_start[i], unit_start[i + 1]) (W first, then H^T); the
-// arithmetic per unit is accumulate_kernel's.
+// arithmetic per unit is finish_sweep_kernel's.
 __global__ void accumulate_batch_kernel(const AccParams *__restrict__ Ps, const int64_t *__restrict__ unit_start,
                                         int n)
 {
@@ -78,14 +104,7 @@ __global__ void accumulate_batch_kernel(const AccParams *__restrict__ Ps, const 
             s = P.sH;
             s2 = P.sH2;
         }
-        const float4 v = x[u];
-        double2 *ps = reinterpret_cast<double2 *>(s) + 2 * u;
-        double2 *ps2 = reinterpret_cast<double2 *>(s2) + 2 * u;
-        double2 p0 = ps[0], p1 = ps[1], q0 = ps2[0], q1 = ps2[1];
-        const double a0 = v.x, a1 = v.y, a2 = v.z, a3 = v.w;
-        p0.x += a0; p0.y += a1; p1.x += a2; p1.y += a3;
-        q0.x += a0 * a0; q0.y += a1 * a1; q1.x += a2 * a2; q1.y += a3 * a3;
-        ps[0] = p0; ps[1] = p1; ps2[0] = q0; ps2[1] = q1;
+        accumulate4(x[u], reinterpret_cast<double2 *>(s) + 2 * u, reinterpret_cast<double2 *>(s2) + 2 * u);
     }
 }
 
@@ -97,11 +116,6 @@ __global__ void t_batch_kernel(const AccParams *__restrict__ Ps, int n, int mode
         if (mode == 0) *P.t_dev = P.t0;
         else *P.t_dev += P.B;
     }
-}
-
-__global__ void advance_t_kernel(int64_t *t, int64_t by)
-{
-    if (threadIdx.x == 0 && blockIdx.x == 0) *t += by;
 }
 
 __device__ double beta_div(double v, double mu, double p)
@@ -307,13 +321,28 @@ reduce_dense_tiled_kernel(int mode, const float *__restrict__ V, int64_t ldv, in
 
 int reduce_blocks() { return kRedBlocks; }
 
-psgld_status launch_accumulate(psgld_ctx *c, cudaStream_t st)
+psgld_status launch_finish_sweep(psgld_ctx *c, bool acc, int64_t by, cudaStream_t st)
 {
-    const int64_t nW4 = c->I * c->ldk / 4, nH4 = c->J * c->ldk / 4;
-    accumulate_kernel<<<(unsigned)std::min<int64_t>((nW4 + 255) / 256, 152 * 16), 256, 0, st>>>(
-        reinterpret_cast<const float4 *>(c->W[c->wcur]), nW4, c->sW.s, c->sW.s2);
-    accumulate_kernel<<<(unsigned)std::min<int64_t>((nH4 + 255) / 256, 152 * 16), 256, 0, st>>>(
-        reinterpret_cast<const float4 *>(c->Ht[c->hcur]), nH4, c->sH.s, c->sH.s2);
+    FinishParams P{};
+    P.x[0] = reinterpret_cast<const float4 *>(c->W[c->wcur]);
+    P.x[1] = reinterpret_cast<const float4 *>(c->Ht[c->hcur]);
+    P.s[0] = c->sW.s;
+    P.s[1] = c->sH.s;
+    P.s2[0] = c->sW.s2;
+    P.s2[1] = c->sH.s2;
+    P.n0 = acc ? c->I * c->ldk / 4 : 0;
+    P.n = acc ? P.n0 + c->J * c->ldk / 4 : 0;
+    P.t = by > 0 ? c->t_dev : nullptr;
+    P.by = by;
+    const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>((P.n + 255) / 256, 152 * 16));
+    finish_sweep_kernel<<<grid, P.n ? 256 : 32, 0, st>>>(P);
+    PSGLD_CK(c, cudaGetLastError());
+    return PSGLD_OK;
+}
+
+psgld_status launch_eps_table(psgld_ctx *c, cudaStream_t st)
+{
+    eps_table_kernel<<<1, 64, 0, st>>>(c->t_dev, c->B, c->opt.eps_a, c->opt.eps_b, c->eps_tab);
     PSGLD_CK(c, cudaGetLastError());
     return PSGLD_OK;
 }
@@ -353,13 +382,6 @@ psgld_status launch_t_batch(psgld_ctx *c0, const void *params, int n, int mode, 
 {
     t_batch_kernel<<<(n + 255) / 256, 256, 0, st>>>(static_cast<const AccParams *>(params), n, mode);
     PSGLD_CK(c0, cudaGetLastError());
-    return PSGLD_OK;
-}
-
-psgld_status launch_advance_t(psgld_ctx *c, int64_t by, cudaStream_t st)
-{
-    advance_t_kernel<<<1, 32, 0, st>>>(c->t_dev, by);
-    PSGLD_CK(c, cudaGetLastError());
     return PSGLD_OK;
 }
 
