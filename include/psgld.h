@@ -94,9 +94,9 @@ typedef struct {
     int32_t dense_path;       /* dense V on the tensor cores, read when data is set:
                                * 0: off (dense V becomes the sparse layout of all
                                *    I*J entries, FP32 gather path);
-                               * 1: on, kernel chosen by shape: single-pass for
-                               *    blocks of at most 128 rows with K <= 128,
-                               *    else two-sided;
+                               * 1: on, kernel chosen: two-sided (single-pass with
+                               *    dense_fp8, and for blocks of at most 128 rows
+                               *    with K <= 128 when V's tiles find no memory);
                                * 2: on, two-sided kernel (K <= 256);
                                * 3: on, single-pass kernel (K <= 128, FP32 V) */
     int32_t dense_v_bf16;     /* 1: the two-sided kernel keeps V in BF16 */

@@ -1094,7 +1094,7 @@ int64_t psgld_estimate_device_bytes(int64_t I, int64_t J, int32_t K, int32_t B, 
     bytes += I * J * 4;   // the FP32 copy of V
     const int64_t maxI = cdiv(I, B), maxJ = cdiv(J, B);
     const int64_t mtiles = cdiv(maxI, 128);
-    const bool two = dense_path == 2 || (dense_path == 1 && (dense_v_bf16 || K > 128 || mtiles > 1));
+    const bool two = dense_path != 3;
     if (!two) {
         if (mtiles > 1) bytes += mtiles * J * ldk * 4;
         return bytes;

@@ -2332,13 +2332,18 @@ psgld_status prepare_dense(psgld_ctx *c, cudaStream_t st)
     if (!dense_supported(c->K)) return fail(c, PSGLD_ERR_ARG, "dense tensor-core path supports K <= 256");
     c->mtiles = dense_mtiles(c);
     const bool f8 = c->opt.dense_fp8 != 0;
-    bool two = mode == 2 || (mode == 1 && !f8 && (vb || c->K > 128 || c->mtiles > 1));
     if ((mode == 3 || f8) && (vb || c->K > 128 || mode == 2))
         return fail(c, PSGLD_ERR_ARG, "single-pass dense kernel (and its E4M3 GEMM1): K <= 128, FP32 V");
-    if (!two) {
+    // dense_path 1 takes the two-sided kernel wherever it can: it spreads a
+    // block over a CTA per 128 rows and per 128 columns and overlaps its copies
+    // and MMAs, where the single-pass one walks a block's columns in one CTA.
+    // Part-step of one chain, single-pass and two-sided: 513 x 4000, K = 32,
+    // B = 8: 53.6 and 14.1 us; 513 x 20000, K = 64: 270 and 48; 257 x 500,
+    // K = 16: 13.6 and 9.0; 256 x 256, K = 8, B = 4: 15.4 and 9.3; 1024^2,
+    // K = 128: 31.3 and 12.1; 256 such chains batched, a sweep: 5.48 and 3.85 ms.
+    if (mode == 3 || f8) {
         c->dense_kind = 1;
         const int kp = dense_kp(c->K);
-        const bool f8 = c->opt.dense_fp8 != 0;
         PSGLD_CK(c, cudaFuncSetAttribute(pick_dense(kp, f8), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)dense_smem(kp, f8)));
         c->dense_fp8 = f8 ? 1 : 0;
@@ -2384,6 +2389,21 @@ psgld_status prepare_dense(psgld_ctx *c, cudaStream_t st)
     if (s == PSGLD_OK) s = al((void **)&c->Hsh, (size_t)nH * 2);
     if (s == PSGLD_OK && nE) s = al((void **)&c->Et, (size_t)nE * 2);
     if (s == PSGLD_OK) s = al((void **)&c->tsync, sizeof(int) * (size_t)(2 + B));
+    if (s == PSGLD_ERR_OOM && mode == 1 && !vb && c->K <= 128 && c->mtiles == 1) {
+        // no room for V's tiles: these blocks also run on the single-pass
+        // kernel, which reads V as it is
+        if (cudaStreamSynchronize(st) != cudaSuccess) return cuda_fail(c, cudaGetLastError(), "sync");
+        void **held[] = {&c->VA, &c->VB, (void **)&c->Wsh, (void **)&c->Hsh, (void **)&c->Et};
+        for (void **p : held) {
+            dev_free(c, *p, st);
+            *p = nullptr;
+        }
+        c->dense_kind = 1;
+        const int kp = dense_kp(c->K);
+        PSGLD_CK(c, cudaFuncSetAttribute(pick_dense(kp, false), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)dense_smem(kp, false)));
+        return PSGLD_OK;
+    }
     return s;
 }
 
