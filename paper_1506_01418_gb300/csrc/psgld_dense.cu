@@ -540,6 +540,8 @@ __device__ __forceinline__ void dense_grad_cta(const DenseParams &P, int cta)
 template <int KP, bool F8>
 __global__ void __launch_bounds__(kDenseThreads, 1) dense_grad_kernel(const __grid_constant__ DenseParams P)
 {
+    dev::wait_prior();
+    dev::let_next();
     dense_grad_cta<KP, F8>(P, blockIdx.x);
 }
 
@@ -551,6 +553,8 @@ __global__ void __launch_bounds__(kDenseThreads, 1)
 dense_grad_batch_kernel(const unsigned char *__restrict__ tab, size_t stride, const int *__restrict__ cta_start,
                         int n)
 {
+    dev::wait_prior();
+    dev::let_next();
     const int b = blockIdx.x;
     int lo = 0, hi = n - 1;          // last i with cta_start[i] <= b
     while (lo < hi) {
@@ -830,7 +834,7 @@ __device__ __forceinline__ const Params &ctx_of(const Params &P0, const Src &src
 // The kernel body.  P0 gives what is uniform over the launch (K width,
 // ring depths); each item reads its own context's parameters.
 template <typename VT, int PM, bool BATCH>
-__device__ __forceinline__ void chain_body(const Params &P0, const Src src, const int total_items)
+__device__ __forceinline__ void chain_body(const Params &P0, const Src src, int total_items, const bool late)
 {
     extern __shared__ __align__(1024) unsigned char sm_raw[];
     // the swizzled operand tiles need 1024-byte alignment (1 KB of slack is allocated)
@@ -870,6 +874,10 @@ __device__ __forceinline__ void chain_body(const Params &P0, const Src src, cons
     __syncthreads();
     fence_after();
     const uint32_t tmem = S->tmem;
+    // a late launch's inputs are complete already (launch_dense_batch): it
+    // waits at its end, so that the launch after it waits for both
+    if (!late) dev::wait_prior();
+    dev::let_next();
 
     if (warp == 0) {
         // ---------------- producer (whole warp, lane 0 performs)
@@ -1093,6 +1101,7 @@ __device__ __forceinline__ void chain_body(const Params &P0, const Src src, cons
         __syncwarp();
     }
 
+    if (late) dev::wait_prior();
     fence_before();
     __syncthreads();
     fence_after();
@@ -1112,16 +1121,16 @@ __device__ __forceinline__ void chain_body(const Params &P0, const Src src, cons
 template <typename VT, int PM>
 __global__ void __launch_bounds__(kThreads, 1) chain_kernel(const __grid_constant__ Params P)
 {
-    chain_body<VT, PM, false>(P, Src{nullptr, nullptr, 1, 0}, P.items);
+    chain_body<VT, PM, false>(P, Src{nullptr, nullptr, 1, 0}, P.items, false);
 }
 
 // Many contexts of one K width, V type and power in one persistent launch.
 template <typename VT, int PM>
 __global__ void __launch_bounds__(kThreads, 1)
-chain_batch_kernel(const unsigned char *tab, size_t stride, const int *item_start, int n)
+chain_batch_kernel(const unsigned char *tab, size_t stride, const int *item_start, int n, int late)
 {
     chain_body<VT, PM, true>(*reinterpret_cast<const Params *>(tab), Src{tab, item_start, n, stride},
-                             __ldg(item_start + n));
+                             __ldg(item_start + n), late != 0);
 }
 
 }  // namespace two_sided_rc
@@ -1586,6 +1595,8 @@ __device__ __forceinline__ void chain_body(const Params &P0, const Src src, cons
     __syncthreads();
     fence_after();
     const uint32_t tmem = S->tmem;
+    dev::wait_prior();
+    dev::let_next();
 
     // E buffer use u (a rows-item tile) takes buffer u % 2 for the (u / 2)-th
     // time; item n completes phase n of g_full.
@@ -2209,7 +2220,7 @@ ChainRcFn pick_chain_rc(bool vb, int pm)
     return f[vb ? 1 : 0][pm];
 }
 
-using ChainRcBatchFn = void (*)(const unsigned char *, size_t, const int *, int);
+using ChainRcBatchFn = void (*)(const unsigned char *, size_t, const int *, int, int);
 
 ChainRcBatchFn pick_chain_batch_rc(bool vb, int pm)
 {
@@ -2536,8 +2547,8 @@ static psgld_status launch_rc(psgld_ctx *c, int part, cudaStream_t st)
     int grid = std::min(P.items, sms);
     if (c->opt.max_sms > 0) grid = std::min(grid, c->opt.max_sms);   // leave SMs to other work
     const size_t smem = rc_smem(c->KP, vs, P.stages, P.vstages);
-    pick_chain_rc(c->v_bf16 != 0, P.p_mode)<<<grid, two_sided_rc::kThreads, smem, st>>>(P);
-    PSGLD_CK(c, cudaGetLastError());
+    PSGLD_CK(c, launch_early(!c->opt.profile, pick_chain_rc(c->v_bf16 != 0, P.p_mode), (unsigned)grid,
+                             two_sided_rc::kThreads, smem, st, P));
     return PSGLD_OK;
 }
 
@@ -2551,8 +2562,8 @@ static psgld_status launch_two_sided(psgld_ctx *c, int part, cudaStream_t st)
     int grid = std::min(P.items, sms);
     if (c->opt.max_sms > 0) grid = std::min(grid, c->opt.max_sms);   // leave SMs to other work
     const size_t smem = two_sided_smem(c->KP, P.stages);
-    pick_chain(c->v_bf16 != 0, P.p_mode)<<<grid, two_sided::kThreads, smem, st>>>(P);
-    PSGLD_CK(c, cudaGetLastError());
+    PSGLD_CK(c, launch_early(!c->opt.profile, pick_chain(c->v_bf16 != 0, P.p_mode), (unsigned)grid,
+                             two_sided::kThreads, smem, st, P));
     return PSGLD_OK;
 }
 
@@ -2588,8 +2599,7 @@ psgld_status launch_dense_grad(psgld_ctx *c, int part, cudaStream_t st)
     if (!fn) return fail(c, PSGLD_ERR_ARG, "single-pass dense kernel supports K <= 128");
     DenseParams P;
     fill_dense_params(c, part, P);
-    fn<<<c->B * P.mtiles, kDenseThreads, dense_smem(kp, f8), st>>>(P);
-    PSGLD_CK(c, cudaGetLastError());
+    PSGLD_CK(c, launch_early(!c->opt.profile, fn, (unsigned)(c->B * P.mtiles), kDenseThreads, dense_smem(kp, f8), st, P));
     return PSGLD_OK;
 }
 
@@ -2636,8 +2646,9 @@ int fill_dense_param(const psgld_ctx *c, int part, void *dst, int *first_items)
 }
 
 psgld_status launch_dense_batch(psgld_ctx *c0, int key, const void *params, const int *cta_start, int n,
-                                int total, cudaStream_t st)
+                                int total, bool late, cudaStream_t st)
 {
+    const bool early = !c0->opt.profile;
     const unsigned char *tab = static_cast<const unsigned char *>(params);
     const size_t stride = dense_param_bytes();
     if (key >= 4096 && key < 8192) {
@@ -2656,8 +2667,9 @@ psgld_status launch_dense_batch(psgld_ctx *c0, int key, const void *params, cons
         PSGLD_CK(c0, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c0->device));
         int grid = std::min(total, sms);
         if (c0->opt.batch_ctas > 0) grid = std::min(grid, (int)c0->opt.batch_ctas);
-        if (grid > 0) fn<<<grid, two_sided_rc::kThreads, smem, st>>>(tab, stride, cta_start, n);
-        PSGLD_CK(c0, cudaGetLastError());
+        if (grid > 0)
+            PSGLD_CK(c0, launch_early(early, fn, (unsigned)grid, two_sided_rc::kThreads, smem, st, tab, stride, cta_start,
+                                      n, early && late ? 1 : 0));
         return PSGLD_OK;
     }
     if (key >= 8192) {
@@ -2673,8 +2685,9 @@ psgld_status launch_dense_batch(psgld_ctx *c0, int key, const void *params, cons
         PSGLD_CK(c0, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c0->device));
         int grid = std::min(total, sms);
         if (c0->opt.batch_ctas > 0) grid = std::min(grid, (int)c0->opt.batch_ctas);
-        if (grid > 0) fn<<<grid, two_sided::kThreads, smem, st>>>(tab, stride, cta_start, cta_start + n + 1, n);
-        PSGLD_CK(c0, cudaGetLastError());
+        if (grid > 0)
+            PSGLD_CK(c0, launch_early(early, fn, (unsigned)grid, two_sided::kThreads, smem, st, tab, stride, cta_start,
+                                      cta_start + n + 1, n));
         return PSGLD_OK;
     }
     const int kp = key / 2;
@@ -2683,8 +2696,8 @@ psgld_status launch_dense_batch(psgld_ctx *c0, int key, const void *params, cons
     if (!fn) return fail(c0, PSGLD_ERR_ARG, "single-pass dense kernel supports K <= 128");
     const size_t smem = dense_smem(kp, f8);
     PSGLD_CK(c0, cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    if (total > 0) fn<<<total, kDenseThreads, smem, st>>>(tab, stride, cta_start, n);
-    PSGLD_CK(c0, cudaGetLastError());
+    if (total > 0)
+        PSGLD_CK(c0, launch_early(early, fn, (unsigned)total, kDenseThreads, smem, st, tab, stride, cta_start, n));
     return PSGLD_OK;
 }
 

@@ -30,6 +30,7 @@
 #include <stdint.h>
 
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "../../include/psgld.h"
@@ -177,6 +178,32 @@ void dev_free(psgld_ctx *c, void *p, cudaStream_t st = nullptr);
 void mark_enqueued(psgld_ctx *c, cudaStream_t st);
 cudaError_t wait_enqueued(psgld_ctx *c);
 
+// ---- launches that start early ---------------------------------------------
+// Programmatic dependent launch: the kernel's blocks may become resident
+// while the kernel before it in the stream drains (once all of that one's
+// blocks have called dev::let_next or ended), and wait for its end at
+// dev::wait_prior, so that the launch itself, and what a kernel does before
+// it reads anything, cost nothing between two kernels of a sweep.  Every
+// kernel launched this way calls dev::wait_prior before it touches memory
+// that an earlier kernel writes, or that one reads and it writes.  With
+// `early` false (profiling: events between the kernels) a plain launch.
+template <class... KA, class... A>
+cudaError_t launch_early(bool early, void (*kernel)(KA...), unsigned grid, int threads, size_t smem,
+                         cudaStream_t st, A &&...args)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = early ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+}
+
 // ---- error plumbing ------------------------------------------------------
 psgld_status fail(psgld_ctx *c, psgld_status s, const std::string &msg);
 psgld_status cuda_fail(psgld_ctx *c, cudaError_t e, const char *what);
@@ -254,8 +281,11 @@ psgld_status launch_dense_grad(psgld_ctx *c, int part, cudaStream_t st);
 int dense_batch_key(const psgld_ctx *c);
 size_t dense_param_bytes();
 int fill_dense_param(const psgld_ctx *c, int part, void *dst, int *first_items);
+// late (not the part's first gradient launch): the launch waits for the one
+// before it at its end instead of its start -- the two share nothing, and
+// that one has waited for the update before them.
 psgld_status launch_dense_batch(psgld_ctx *c0, int key, const void *params, const int *cta_start, int n,
-                                int total, cudaStream_t st);
+                                int total, bool late, cudaStream_t st);
 // Update of part `part` at iteration *t_dev + t_add (t_dev: the context's
 // device counter); does not flip the context's buffers.
 size_t upd_param_bytes();
@@ -287,6 +317,13 @@ int bits_for(uint64_t n_values);
 // ---- device helpers -------------------------------------------------------
 namespace psgld {
 namespace dev {
+
+// Waits for the kernels before this one in the stream (launch_early); at once
+// for a plain launch.
+__device__ __forceinline__ void wait_prior() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// The next kernel's blocks may become resident from here on.
+__device__ __forceinline__ void let_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // Philox4x32-10 (Salmon et al., SC'11): ten rounds of two 32x32->64-bit
 // multiplies whose high halves are mixed into the other two words with the

@@ -40,6 +40,7 @@ struct FinishParams {
 
 __global__ void finish_sweep_kernel(const __grid_constant__ FinishParams P)
 {
+    dev::wait_prior();
     if (P.t && blockIdx.x == 0 && threadIdx.x == 0) *P.t += P.by;
     for (int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; a < P.n;
          a += (int64_t)gridDim.x * blockDim.x) {
@@ -335,8 +336,7 @@ psgld_status launch_finish_sweep(psgld_ctx *c, bool acc, int64_t by, cudaStream_
     P.t = by > 0 ? c->t_dev : nullptr;
     P.by = by;
     const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>((P.n + 255) / 256, 152 * 16));
-    finish_sweep_kernel<<<grid, P.n ? 256 : 32, 0, st>>>(P);
-    PSGLD_CK(c, cudaGetLastError());
+    PSGLD_CK(c, launch_early(!c->opt.profile, finish_sweep_kernel, grid, P.n ? 256 : 32, 0, st, P));
     return PSGLD_OK;
 }
 

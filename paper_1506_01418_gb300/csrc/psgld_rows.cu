@@ -356,6 +356,8 @@ __global__ void __launch_bounds__(kThreads, MINB) rows_kernel(const __grid_const
     const int l = lane & (T - 1), team = lane / T;
     const bool in_last = l + (NG - 1) * T < P.ng;
     const int n_heavy = P.side[0].n_heavy + P.side[1].n_heavy;
+    dev::let_next();
+    dev::wait_prior();
     if (P.wait_polls && !gather_wait_check(P, P.side[P.side[0].n_rows ? 0 : 1])) return;
     const Clock clk = read_clock(P.noise);
     Row<T, NG> r;
@@ -659,7 +661,7 @@ psgld_status launch_rows(psgld_ctx *c, int part, int64_t t, const int64_t *t_dev
     P.err = c->kflag;
     P.wait_polls = (uint32_t)c->opt.debug_wait_polls;
     fill_noise(c, part, t, t_dev, t_add, P.noise);
-    if (grid > 0) k.fn<<<(unsigned)grid, kThreads, 0, st>>>(P);
+    if (grid > 0) PSGLD_CK(c, launch_early(!c->opt.profile, k.fn, (unsigned)grid, kThreads, 0, st, P));
     PSGLD_CK(c, cudaGetLastError());
     return PSGLD_OK;
 }

@@ -39,6 +39,7 @@ struct UpdParams {
     StepNoise noise;
     int K, ldk, ngroups;
     uint32_t div_magic;       // ceil(2^32 / ngroups) when item * ngroups < 2^32, else 0
+    int small;                // 1: every index below 2^31 (update_item_dense32)
     int eps_poly;             // 1: eps_t = (a/t)^b computed on the device (no table)
     double eps_a, eps_b;
     int B, sh_kp;             // pieces; shadow tile width (two-sided dense kernel)
@@ -88,6 +89,8 @@ __device__ __forceinline__ void update_item(const UpdParams &P, int64_t item, fl
 
 __global__ void __launch_bounds__(kThreads, 5) update_kernel(const __grid_constant__ UpdParams P)
 {
+    dev::wait_prior();
+    dev::let_next();
     float eps, sd;
     const int64_t t = read_step(P, eps, sd);
     const uint32_t t_lo = (uint32_t)(uint64_t)t, t_hi = (uint32_t)((uint64_t)t >> 32);
@@ -143,6 +146,8 @@ __device__ __forceinline__ void update_item_dense32(const UpdParams &P, uint32_t
 
 __global__ void __launch_bounds__(kThreads, 5) update_kernel_dense32(const __grid_constant__ UpdParams P)
 {
+    dev::wait_prior();
+    dev::let_next();
     float eps, sd;
     const int64_t t = read_step(P, eps, sd);
     const uint32_t t_lo = (uint32_t)(uint64_t)t, t_hi = (uint32_t)((uint64_t)t >> 32);
@@ -218,6 +223,13 @@ static void fill_params(psgld_ctx *c, int part, int64_t t, const int64_t *t_dev,
                        : 0u;
     UP.B = c->B;
     UP.sh_kp = c->KP;
+    // 32-bit arithmetic: items, factor rows, every partial gradient array and
+    // the BF16 shadows within 2^31
+    const int64_t lim = (1ll << 31) - 1;
+    const int64_t sh_elems = c->dense_kind == 2
+        ? (int64_t)c->B * 2 * std::max<int64_t>(c->mt_max, c->nt_max) * 64 * c->KP : 0;
+    UP.small = UP.side[0].items + UP.side[1].items <= lim && std::max(c->I, c->J) * c->ldk <= lim &&
+               (int64_t)std::max(1, c->mtiles) * c->J * c->ldk <= lim && sh_elems <= lim;
 }
 
 psgld_status launch_part_step(psgld_ctx *c, int64_t t, const int64_t *t_dev, int64_t t_add,
@@ -251,18 +263,11 @@ psgld_status launch_part_step(psgld_ctx *c, int64_t t, const int64_t *t_dev, int
         }
         PSGLD_CK(c, cudaGetLastError());
         if (prof) PSGLD_CK(c, cudaEventRecordWithFlags(c->ev_mid[part], st, rec_flags));
-        // the 32-bit update: items, factor rows, every partial gradient
-        // array and the BF16 shadows within 2^31
-        const int64_t lim = (1ll << 31) - 1;
         const int64_t items = UP.side[0].items + UP.side[1].items;
-        const int64_t sh_elems = c->dense_kind == 2
-            ? (int64_t)B * 2 * std::max<int64_t>(c->mt_max, c->nt_max) * 64 * c->KP : 0;
-        const bool dense32 = items <= lim && std::max(c->I, c->J) * c->ldk <= lim &&
-                             (int64_t)std::max(1, c->mtiles) * c->J * c->ldk <= lim && sh_elems <= lim;
         const int grid = (int)std::min<int64_t>((items + kThreads - 1) / kThreads, 152 * 16);
         if (grid > 0) {
-            if (dense32) update_kernel_dense32<<<grid, kThreads, 0, st>>>(UP);
-            else update_kernel<<<grid, kThreads, 0, st>>>(UP);
+            PSGLD_CK(c, launch_early(!prof, UP.small ? update_kernel_dense32 : update_kernel, (unsigned)grid, kThreads,
+                                     0, st, UP));
         }
     }
     PSGLD_CK(c, cudaGetLastError());
@@ -279,31 +284,49 @@ namespace {
 
 // ---- many contexts in one update launch ------------------------------------
 
+// Block b takes a contiguous run of the items of all contexts, so that it
+// looks a context up once and then steps from one to the next (256 chains of
+// 513 x 200-5000, K = 32: a launch 115 to 91 us, with 32-bit index arithmetic
+// where a context's arrays allow it).
 __global__ void __launch_bounds__(kThreads, 4)
 update_batch_kernel(const UpdParams *__restrict__ Ps, const int64_t *__restrict__ item_start, int n)
 {
+    dev::wait_prior();
+    dev::let_next();
     const int64_t total = __ldg(item_start + n);
-    const int64_t stride = (int64_t)gridDim.x * kThreads;
-    int ci = -1;
-    float eps = 0.f, sd = 0.f;
-    uint32_t t_lo = 0, t_hi = 0;
-    for (int64_t a = blockIdx.x * (int64_t)kThreads + threadIdx.x; a < total; a += stride) {
-        if (ci < 0 || __ldg(item_start + ci + 1) <= a) {
-            int lo = ci < 0 ? 0 : ci, hi = n - 1;   // last i with item_start[i] <= a
-            while (lo < hi) {
-                const int mid = (lo + hi + 1) >> 1;
-                if (__ldg(item_start + mid) <= a) lo = mid; else hi = mid - 1;
-            }
-            ci = lo;
-            const UpdParams &P = Ps[ci];
-            const int64_t t = read_step(P, eps, sd);
-            t_lo = (uint32_t)(uint64_t)t;
-            t_hi = (uint32_t)((uint64_t)t >> 32);
+    const int64_t per = ((total + gridDim.x - 1) / gridDim.x + kThreads - 1) / kThreads * kThreads;
+    const int64_t from = blockIdx.x * per, to = from + per < total ? from + per : total;
+    if (from >= to) return;
+    int ci;
+    {
+        int lo = 0, hi = n - 1;   // last i with item_start[i] <= from
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (__ldg(item_start + mid) <= from) lo = mid; else hi = mid - 1;
         }
+        ci = lo;
+    }
+    for (int64_t begin = from; begin < to; ++ci) {   // one context's part of the run
+        const int64_t first = __ldg(item_start + ci), next = __ldg(item_start + ci + 1);
+        const int64_t end = next < to ? next : to;
         const UpdParams &P = Ps[ci];
-        const int64_t local = a - __ldg(item_start + ci);
-        if (local < P.side[0].items) update_item<0>(P, local, eps, sd, t_lo, t_hi);
-        else update_item<1>(P, local - P.side[0].items, eps, sd, t_lo, t_hi);
+        float eps, sd;
+        const int64_t t = read_step(P, eps, sd);
+        const uint32_t t_lo = (uint32_t)(uint64_t)t, t_hi = (uint32_t)((uint64_t)t >> 32);
+        const int64_t n0 = P.side[0].items;
+        if (P.small) {
+            const uint32_t w = (uint32_t)n0;
+            for (uint32_t a = (uint32_t)(begin - first) + threadIdx.x; a < (uint32_t)(end - first); a += kThreads) {
+                if (a < w) update_item_dense32<0>(P, a, eps, sd, t_lo, t_hi);
+                else update_item_dense32<1>(P, a - w, eps, sd, t_lo, t_hi);
+            }
+        } else {
+            for (int64_t a = begin - first + threadIdx.x; a < end - first; a += kThreads) {
+                if (a < n0) update_item<0>(P, a, eps, sd, t_lo, t_hi);
+                else update_item<1>(P, a - n0, eps, sd, t_lo, t_hi);
+            }
+        }
+        begin = end;
     }
 }
 
@@ -329,8 +352,8 @@ psgld_status launch_update_batch(psgld_ctx *c0, const void *params, const int64_
     const int64_t cap = c0->opt.batch_update_blocks > 0 ? c0->opt.batch_update_blocks : 152 * 16;
     const int grid = (int)std::min<int64_t>((total_items + kThreads - 1) / kThreads, cap);
     if (grid > 0)
-        update_batch_kernel<<<grid, kThreads, 0, st>>>(static_cast<const UpdParams *>(params), item_start, n);
-    PSGLD_CK(c0, cudaGetLastError());
+        PSGLD_CK(c0, launch_early(!c0->opt.profile, update_batch_kernel, (unsigned)grid, kThreads, 0, st,
+                                  static_cast<const UpdParams *>(params), item_start, n));
     return PSGLD_OK;
 }
 
