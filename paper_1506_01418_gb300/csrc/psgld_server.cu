@@ -116,7 +116,12 @@ bool setup(psgld_server *s, Job *j)
     const psgld_job &q = j->spec;
     psgld_ctx *c = nullptr;
     psgld_status st = psgld::create_context(q.I, q.J, q.K, q.B, q.tweedie_p, q.phi, &q.prior, &s->allocator, &c);
-    if (st == PSGLD_OK) st = psgld_set_options(c, &q.options);
+    // direct launches: a stream capture on this thread would make another
+    // thread's cudaDeviceSynchronize fail while it lasts, and the list of
+    // jobs rarely stays long enough for its graph to be replayed
+    psgld_options options = q.options;
+    options.use_graphs = 0;
+    if (st == PSGLD_OK) st = psgld_set_options(c, &options);
     if (st == PSGLD_OK) st = psgld_set_data_dense(c, q.V_dev, q.ldv, s->adm);
     if (st == PSGLD_OK) st = psgld_set_factors(c, q.W0_dev, q.Ht0_dev, s->adm);
     if (st == PSGLD_OK && (cudaEventCreateWithFlags(&j->ready, cudaEventDisableTiming) != cudaSuccess ||
