@@ -462,18 +462,29 @@ psgld_status psgld_set_data_coo(psgld_ctx *c, int64_t nnz, const int32_t *i, con
     if (nnz > 0 && (!i || !j || !v)) return fail(c, PSGLD_ERR_ARG, "null entry array");
     cudaStream_t st = (cudaStream_t)stream;
     destroy_graphs(c);
+    // entries already on this device are read where they are
+    auto here = [&](const void *p) {
+        cudaPointerAttributes at{};
+        const bool dev = p && cudaPointerGetAttributes(&at, p) == cudaSuccess && at.type == cudaMemoryTypeDevice &&
+                         at.device == c->device;
+        if (!dev) cudaGetLastError();
+        return dev;
+    };
     int32_t *di = nullptr, *dj = nullptr;
     float *dv = nullptr;
-    psgld_status s = alloc(c, &di, nnz, false, st);
-    if (s == PSGLD_OK) s = alloc(c, &dj, nnz, false, st);
-    if (s == PSGLD_OK) s = alloc(c, &dv, nnz, false, st);
-    if (s == PSGLD_OK && nnz > 0) {
-        cudaError_t e = cudaMemcpyAsync(di, i, sizeof(int32_t) * nnz, cudaMemcpyDefault, st);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(dj, j, sizeof(int32_t) * nnz, cudaMemcpyDefault, st);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(dv, v, sizeof(float) * nnz, cudaMemcpyDefault, st);
+    psgld_status s = PSGLD_OK;
+    auto stage = [&](auto **copy, auto *&src) {
+        if (s != PSGLD_OK || nnz == 0 || here(src)) return;
+        s = alloc(c, copy, nnz, false, st);
+        if (s != PSGLD_OK) return;
+        const cudaError_t e = cudaMemcpyAsync(*copy, src, sizeof(**copy) * nnz, cudaMemcpyDefault, st);
         if (e != cudaSuccess) s = cuda_fail(c, e, "copy entries");
-    }
-    if (s == PSGLD_OK) s = build_layout(c, nnz, di, dj, dv, st);
+        src = *copy;
+    };
+    stage(&di, i);
+    stage(&dj, j);
+    stage(&dv, v);
+    if (s == PSGLD_OK) s = build_layout(c, nnz, i, j, v, st);
     if (s == PSGLD_OK) s = zero_posterior(c, st);
     if (s == PSGLD_OK) {
         cudaError_t e = cudaStreamSynchronize(st);

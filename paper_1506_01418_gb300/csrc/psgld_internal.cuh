@@ -92,6 +92,9 @@ struct psgld_ctx {
     int64_t N = 0;
     std::vector<int64_t> part_n;     // observed entries of each part
     psgld::SideLayout side[2];       // 0: rows of W (CSR), 1: rows of Ht (CSC)
+    void *layout_mem = nullptr;      // one allocation with both sides' arrays
+    size_t layout_bytes = 0;
+    void *chunk_mem = nullptr;       // ... with the heavy rows' sums and counters
     bool dense = false;              // data kept dense for the tensor-core path
     float *Vd = nullptr;             // I x ldv fp32 (dense path)
     int64_t ldv = 0;

@@ -10,10 +10,21 @@
 // Both are produced by a stable LSD radix sort written here (8-bit digits,
 // per-tile histograms, a global exclusive scan and a stable scatter whose
 // in-tile ranks come from warp match/ballot), so the order is exact and
-// repeatable.  The A side's entries also record their row of W, for the
-// reductions over all entries, and both sides list, per part, the rows with
-// many entries, which the part-step gives more lanes.
+// repeatable.  What is sorted are whole entries (a 32-bit key, the other
+// index, the value), so the last pass writes the layout itself.  The A side
+// of entries that come in row-major order needs the parts' digits alone
+// (stable: rows and columns stay in order within a part), one pass for up to
+// 256 parts; other entries take the columns' digits, then those of s*I + i.
+// The B side starts from the A side, whose parts hold their rows in order, so
+// the digits of s*J + j are enough.  10^7 entries, 70000 x 10000, B = 32: 4
+// passes, where sorting 64-bit (part, row, column) keys with a permutation
+// took 5 for each side and gathered the entries through it afterwards; load,
+// factors and a part-step 3.99 to 1.54 ms.
+// The A side's entries also keep their row of W, for the reductions over all
+// entries, and both sides list, per part, the rows with many entries, which
+// the part-step gives more lanes.
 #include <algorithm>
+#include <utility>
 
 #include "psgld_internal.cuh"
 
@@ -137,58 +148,84 @@ __global__ void scan_tiles(const uint32_t *__restrict__ in, int64_t n,
 // ---- radix sort -----------------------------------------------------------
 
 constexpr int kSortThreads = 256;
-constexpr int kSortItems = 8;
-constexpr int kSortTile = kSortThreads * kSortItems;  // 2048 keys per CTA
+constexpr int kSortItems = 16;
+constexpr int kSortTile = kSortThreads * kSortItems;  // 4096 entries per CTA
 constexpr int kSortWarps = kSortThreads / 32;
 
-__global__ void radix_hist(const uint64_t *__restrict__ keys, int64_t n, int shift,
-                           uint32_t *__restrict__ hist, int64_t ntiles)
+// Entries as three arrays: key, other index, value.
+struct Entries {
+    const uint32_t *key, *other;
+    const float *val;
+};
+
+// Digit of an entry: 8 bits at `shift` of its key divided by `div`, or
+// (by_other) of its other index.
+struct Digit {
+    uint32_t div;
+    int shift, by_other;
+
+    __device__ __forceinline__ uint32_t of(uint32_t key, uint32_t other) const
+    {
+        const uint32_t x = by_other ? other : div > 1 ? key / div : key;
+        return (x >> shift) & 255u;
+    }
+};
+
+__global__ void radix_hist(const Entries in, int64_t n, const Digit D, uint32_t *__restrict__ hist, int64_t ntiles)
 {
     __shared__ uint32_t h[256];
     h[threadIdx.x] = 0;
     __syncthreads();
     const int64_t base = (int64_t)blockIdx.x * kSortTile;
-    for (int k = threadIdx.x; k < kSortTile; k += kSortThreads)
-        if (base + k < n) atomicAdd(&h[(keys[base + k] >> shift) & 255u], 1u);
+    const uint32_t *src = D.by_other ? in.other : in.key;
+    for (int k = threadIdx.x; k < kSortTile; k += kSortThreads) {
+        const bool ok = base + k < n;
+        const uint32_t x = ok ? __ldg(src + base + k) : 0u;
+        const uint32_t d = ok ? D.of(x, x) : 256u;
+        // equal digits of a warp count once (runs of one part or of one row's
+        // high digit would serialise on one counter)
+        const unsigned peers = __match_any_sync(0xffffffffu, d);
+        if (ok && (threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(&h[d], (uint32_t)__popc(peers));
+    }
     __syncthreads();
     hist[(int64_t)threadIdx.x * ntiles + blockIdx.x] = h[threadIdx.x];
 }
 
-// Stable scatter.  Warp w of the tile owns positions [w*256, (w+1)*256);
-// item m of lane l is position w*256 + m*32 + l, so (w, m, l) order is
+// Stable scatter.  Warp w of the tile owns positions [w*512, (w+1)*512);
+// item m of lane l is position w*512 + m*32 + l, so (w, m, l) order is
 // position order.  Ranks among equal digits come from __match_any_sync.
-__global__ void radix_scatter(const uint64_t *__restrict__ kin, const uint32_t *__restrict__ vin,
-                              int64_t n, int shift, const uint32_t *__restrict__ offs,
-                              int64_t ntiles, uint64_t *__restrict__ kout,
-                              uint32_t *__restrict__ vout)
+__global__ void __launch_bounds__(kSortThreads)
+radix_scatter(const Entries in, int64_t n, const Digit D, const uint32_t *__restrict__ offs, int64_t ntiles,
+              uint32_t *__restrict__ key_out, uint32_t *__restrict__ other_out, float *__restrict__ val_out)
 {
     __shared__ uint32_t wcnt[kSortWarps][256];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int d = threadIdx.x; d < kSortWarps * 256; d += kSortThreads) (&wcnt[0][0])[d] = 0;
     __syncthreads();
-    const int64_t base = (int64_t)blockIdx.x * kSortTile + warp * 256;
+    const int64_t base = (int64_t)blockIdx.x * kSortTile + warp * (32 * kSortItems);
     const uint32_t lt = (1u << lane) - 1u;
-    uint64_t key[kSortItems];
-    uint32_t val[kSortItems], rank[kSortItems];
-    int dig[kSortItems];
+    uint32_t key[kSortItems], other[kSortItems], at[kSortItems];   // at: rank << 9 | digit
 #pragma unroll
     for (int m = 0; m < kSortItems; ++m) {
         const int64_t pos = base + m * 32 + lane;
-        const bool ok = pos < n;
-        key[m] = ok ? kin[pos] : 0ull;
-        val[m] = ok ? vin[pos] : 0u;
-        dig[m] = ok ? (int)((key[m] >> shift) & 255u) : 256 + lane;  // invalid: unique
-        const unsigned peers = __match_any_sync(0xffffffffu, dig[m]);
-        const uint32_t before = ok ? wcnt[warp][dig[m]] : 0u;
-        rank[m] = before + __popc(peers & lt);
+        key[m] = pos < n ? __ldg(in.key + pos) : 0u;
+        other[m] = pos < n ? __ldg(in.other + pos) : 0u;
+    }
+#pragma unroll
+    for (int m = 0; m < kSortItems; ++m) {
+        const bool ok = base + m * 32 + lane < n;
+        const uint32_t d = ok ? D.of(key[m], other[m]) : 256u;
+        const unsigned peers = __match_any_sync(0xffffffffu, d);
+        const uint32_t before = ok ? wcnt[warp][d] : 0u;
+        at[m] = ((before + __popc(peers & lt)) << 9) | d;
         __syncwarp();
-        if (ok && (peers & lt) == 0) wcnt[warp][dig[m]] = before + __popc(peers);
+        if (ok && (peers & lt) == 0) wcnt[warp][d] = before + __popc(peers);
         __syncwarp();
     }
     __syncthreads();
-    {   // exclusive prefix over warps, one digit per thread
+    {   // per digit (one a thread): where each warp's entries go
         const int d = threadIdx.x;
-        uint32_t run = 0;
+        uint32_t run = offs[(int64_t)d * ntiles + blockIdx.x];
         for (int w = 0; w < kSortWarps; ++w) {
             const uint32_t c = wcnt[w][d];
             wcnt[w][d] = run;
@@ -198,62 +235,70 @@ __global__ void radix_scatter(const uint64_t *__restrict__ kin, const uint32_t *
     __syncthreads();
 #pragma unroll
     for (int m = 0; m < kSortItems; ++m) {
-        if (dig[m] < 256) {
-            const uint32_t dst = offs[(int64_t)dig[m] * ntiles + blockIdx.x] + wcnt[warp][dig[m]] + rank[m];
-            kout[dst] = key[m];
-            vout[dst] = val[m];
+        const uint32_t d = at[m] & 511u;
+        if (d < 256u) {
+            const uint32_t dst = wcnt[warp][d] + (at[m] >> 9);
+            key_out[dst] = key[m];
+            other_out[dst] = other[m];
+            val_out[dst] = __ldg(in.val + base + m * 32 + lane);
         }
     }
 }
 
 // ---- layout kernels ---------------------------------------------------------
 
-__device__ __forceinline__ int64_t piece_of(int64_t x, int64_t n, int B)
+// largest r with floor(r n / B) <= x; B n < 2^31 (checked at create)
+__device__ __forceinline__ uint32_t piece_of(uint32_t x, uint32_t n, uint32_t B) { return ((x + 1u) * B - 1u) / n; }
+
+// Checks the entries (flag: 1 index out of range, 2 value, 8 not in strict
+// row-major order) and writes their slots of the A side, s*I + i.
+__global__ void validate_and_key(int64_t nnz, const int32_t *__restrict__ ii, const int32_t *__restrict__ jj,
+                                 const float *__restrict__ vv, uint32_t I, uint32_t J, uint32_t B, int nonneg,
+                                 uint32_t *__restrict__ key, int *flag)
 {
-    // largest r with floor(r n / B) <= x
-    return ((x + 1) * B - 1) / n;
+    int bad = 0;
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nnz;
+         e += (int64_t)gridDim.x * blockDim.x) {
+        const uint32_t i = (uint32_t)ii[e], j = (uint32_t)jj[e];
+        const float v = vv[e];
+        if (i >= I || j >= J) { bad |= 1; continue; }
+        if (!isfinite(v) || (nonneg && v < 0.0f)) bad |= 2;
+        if (e > 0) {
+            const uint32_t ip = (uint32_t)ii[e - 1], jp = (uint32_t)jj[e - 1];
+            if (!(ip < i || (ip == i && jp < j))) bad |= 8;
+        }
+        const uint32_t rp = piece_of(i, I, B), cp = piece_of(j, J, B);
+        key[e] = (cp >= rp ? cp - rp : cp + B - rp) * I + i;
+    }
+    bad = __reduce_or_sync(0xffffffffu, bad);
+    if (bad && (threadIdx.x & 31) == 0) atomicOr(flag, bad);
 }
 
-__global__ void validate_and_key(int64_t nnz, const int32_t *__restrict__ ii,
-                                 const int32_t *__restrict__ jj, const float *__restrict__ vv,
-                                 int64_t I, int64_t J, int B, int nonneg, int bitsI, int bitsJ,
-                                 uint64_t *__restrict__ keyA, uint64_t *__restrict__ keyB,
-                                 uint32_t *__restrict__ valA, uint32_t *__restrict__ valB,
-                                 int *flag)
+// The B side's slots s*J + j and rows i from the A side's order.
+__global__ void key_columns(int64_t nnz, const uint32_t *__restrict__ keyA, const uint32_t *__restrict__ jA, uint32_t I,
+                            uint32_t J, uint32_t *__restrict__ keyB, uint32_t *__restrict__ iB)
 {
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nnz;
          e += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t i = ii[e], j = jj[e];
-        const float v = vv[e];
-        if (i < 0 || i >= I || j < 0 || j >= J) { atomicOr(flag, 1); continue; }
-        if (!isfinite(v) || (nonneg && v < 0.0f)) atomicOr(flag, 2);
-        const int64_t rp = piece_of(i, I, B), cp = piece_of(j, J, B);
-        const int64_t s = (cp - rp + B) % B;
-        keyA[e] = ((uint64_t)(s * I + i) << bitsJ) | (uint64_t)j;
-        keyB[e] = ((uint64_t)(s * J + j) << bitsI) | (uint64_t)i;
-        valA[e] = (uint32_t)e;
-        valB[e] = (uint32_t)e;
+        const uint32_t k = keyA[e], s = k / I;
+        keyB[e] = s * J + jA[e];
+        iB[e] = k - s * I;
     }
 }
 
-// Gather sorted entries; flag duplicates; fill the slot pointer array.
-__global__ void finish_side(int64_t nnz, const uint64_t *__restrict__ key,
-                            const uint32_t *__restrict__ perm, const int32_t *__restrict__ other,
-                            const float *__restrict__ vv, int bits_other, int64_t nslots,
-                            int64_t n_rows, int32_t *__restrict__ idx, float *__restrict__ val,
-                            int32_t *__restrict__ own, int32_t *__restrict__ ptr, int *flag)
+// The slots' first entries; duplicates flagged (4); the entries' own rows.
+__global__ void finish_side(int64_t nnz, const uint32_t *__restrict__ key, const uint32_t *__restrict__ other,
+                            uint32_t nslots, uint32_t n_rows, int32_t *__restrict__ own, int32_t *__restrict__ ptr,
+                            int *flag)
 {
     for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p <= nnz;
          p += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t slot = p < nnz ? (int64_t)(key[p] >> bits_other) : nslots;
-        const int64_t prev = p > 0 ? (int64_t)(key[p - 1] >> bits_other) : -1;
-        for (int64_t s = prev + 1; s <= slot; ++s) ptr[s] = (int32_t)p;
+        const uint32_t slot = p < nnz ? key[p] : nslots;
+        const uint32_t from = p > 0 ? key[p - 1] + 1u : 0u;
+        for (uint32_t s = from; s <= slot; ++s) ptr[s] = (int32_t)p;
         if (p < nnz) {
-            const uint32_t e = perm[p];
-            idx[p] = other[e];
-            val[p] = vv[e];
             if (own) own[p] = (int32_t)(slot % n_rows);
-            if (p > 0 && key[p] == key[p - 1]) atomicOr(flag, 4);
+            if (p > 0 && from == slot + 1u && other[p] == other[p - 1]) atomicOr(flag, 4);
         }
     }
 }
@@ -296,17 +341,22 @@ int grid_for(int64_t n, int threads)
     return (int)std::max<int64_t>(1, std::min<int64_t>(g, 152 * 32));
 }
 
-template <typename T>
-psgld_status dmalloc(psgld_ctx *c, T **p, int64_t n)
-{
-    if (n <= 0) n = 1;
-    // whole 256-byte granules, so that 16-byte-rounded bulk prefetches of any
-    // sub-range stay inside the allocation
-    const size_t bytes = (sizeof(T) * (size_t)n + 255) & ~size_t(255);
-    *p = static_cast<T *>(dev_alloc(c, bytes, nullptr));
-    if (!*p) return fail(c, PSGLD_ERR_OOM, "device allocation of " + std::to_string(sizeof(T) * n) + " bytes failed");
-    return PSGLD_OK;
-}
+// Several arrays in one allocation: sizes first, then the addresses.
+struct Arena {
+    size_t bytes = 0;
+    std::vector<std::pair<void **, size_t>> parts;
+
+    template <typename T>
+    void add(T **p, int64_t n)
+    {
+        parts.emplace_back(reinterpret_cast<void **>(p), bytes);
+        bytes += (sizeof(T) * (size_t)std::max<int64_t>(n, 1) + 255) & ~size_t(255);
+    }
+    void place(void *base) const
+    {
+        for (const auto &q : parts) *q.first = static_cast<unsigned char *>(base) + q.second;
+    }
+};
 
 // Exclusive scan of n uint32 values (in -> out, out has n+1 entries; out[n]
 // is the total).  tmp needs ceil(n / kScanTile) + 1 entries.
@@ -321,21 +371,36 @@ psgld_status exclusive_scan(psgld_ctx *c, const uint32_t *in, uint32_t *out, int
     return PSGLD_OK;
 }
 
-psgld_status radix_sort(psgld_ctx *c, uint64_t *&k0, uint32_t *&v0, uint64_t *&k1,
-                        uint32_t *&v1, int64_t n, int bits, uint32_t *hist, uint32_t *hist_scan,
-                        uint32_t *tmp, cudaStream_t st)
+// The digits of one sort, lowest first.
+std::vector<Digit> digits(uint32_t div, int bits, int by_other)
+{
+    std::vector<Digit> d;
+    for (int shift = 0; shift < std::max(bits, 1); shift += 8) d.push_back({div, shift, by_other});
+    return d;
+}
+
+// Sorts by the given digits: from `in` through the two scratch sets, the last
+// pass's other index and value to `other_out` and `val_out`; returns the
+// sorted keys in *key_out (one of the scratch arrays).
+psgld_status radix_sort(psgld_ctx *c, Entries in, const std::vector<Digit> &ds, int64_t n, uint32_t *const key[2],
+                        uint32_t *const other[2], float *const val[2], uint32_t *other_out, float *val_out,
+                        uint32_t *hist, uint32_t *hist_scan, uint32_t *tmp, const uint32_t **key_out, cudaStream_t st)
 {
     const int64_t ntiles = std::max<int64_t>(1, (n + kSortTile - 1) / kSortTile);
-    for (int shift = 0; shift < bits; shift += 8) {
-        radix_hist<<<(unsigned)ntiles, kSortThreads, 0, st>>>(k0, n, shift, hist, ntiles);
+    int to = in.key == key[0] ? 1 : 0;
+    for (size_t p = 0; p < ds.size(); ++p) {
+        const bool end = p + 1 == ds.size();
+        radix_hist<<<(unsigned)ntiles, kSortThreads, 0, st>>>(in, n, ds[p], hist, ntiles);
         psgld_status s = exclusive_scan(c, hist, hist_scan, 256 * ntiles, tmp, st);
         if (s != PSGLD_OK) return s;
-        radix_scatter<<<(unsigned)ntiles, kSortThreads, 0, st>>>(k0, v0, n, shift, hist_scan,
-                                                                 ntiles, k1, v1);
+        uint32_t *o = end ? other_out : other[to];
+        float *v = end ? val_out : val[to];
+        radix_scatter<<<(unsigned)ntiles, kSortThreads, 0, st>>>(in, n, ds[p], hist_scan, ntiles, key[to], o, v);
         PSGLD_CK(c, cudaGetLastError());
-        std::swap(k0, k1);
-        std::swap(v0, v1);
+        in = {key[to], o, v};
+        to ^= 1;
     }
+    *key_out = in.key;
     return PSGLD_OK;
 }
 
@@ -346,12 +411,11 @@ void free_layout(psgld_ctx *c)
     // work that reads the layouts must be finished before they are handed back
     wait_enqueued(c);
     if (c->capture_stream) cudaStreamSynchronize(c->capture_stream);
-    for (auto &sd : c->side) {
-        dev_free(c, sd.ptr); dev_free(c, sd.idx); dev_free(c, sd.val); dev_free(c, sd.own);
-        dev_free(c, sd.mid); dev_free(c, sd.heavy);
-        dev_free(c, sd.partial); dev_free(c, sd.arrived);
-        sd = SideLayout{};
-    }
+    for (auto &sd : c->side) sd = SideLayout{};
+    dev_free(c, c->layout_mem);
+    dev_free(c, c->chunk_mem);
+    c->layout_mem = c->chunk_mem = nullptr;
+    c->layout_bytes = 0;
     dev_free(c, c->Vd);
     dev_free(c, c->hpart);
     dev_free(c, c->VA);
@@ -379,113 +443,156 @@ void free_layout(psgld_ctx *c)
 psgld_status build_layout(psgld_ctx *c, int64_t nnz, const int32_t *i_dev, const int32_t *j_dev,
                           const float *v_dev, cudaStream_t st)
 {
+    // the memory of the layout before stays when it fits this one
+    void *kept = c->layout_mem;
+    const size_t kept_bytes = c->layout_bytes;
+    c->layout_mem = nullptr;
     free_layout(c);
-    const int64_t I = c->I, J = c->J;
+    const int64_t I = c->I, J = c->J, n = nnz;
     const int B = c->B;
-    const int bitsI = bits_for((uint64_t)I), bitsJ = bits_for((uint64_t)J);
-    const int bitsA = bits_for((uint64_t)(B * I)) + bitsJ;
-    const int bitsB = bits_for((uint64_t)(B * J)) + bitsI;
-    const int64_t n = nnz;
     c->light_row = light_row_for(I + J);
 
-    uint64_t *kA = nullptr, *kB = nullptr, *kt = nullptr;
-    uint32_t *pA = nullptr, *pB = nullptr, *pt = nullptr;
-    uint32_t *hist = nullptr, *hscan = nullptr, *tmp = nullptr;
     const int64_t ntiles = std::max<int64_t>(1, (n + kSortTile - 1) / kSortTile);
     const int64_t nslots_max = (int64_t)B * std::max(I, J);
     const int64_t scan_n = std::max<int64_t>(256 * ntiles + 1, nslots_max + 1);
     const int64_t tmp_n = (scan_n + kScanTile - 1) / kScanTile + 2;
-    psgld_status s = PSGLD_OK;
-    std::vector<void *> scratch;
+    uint32_t *key[2], *other[2], *hist, *hscan, *tmp;
+    float *val[2];
+    int64_t *offs_dev;   // starts of the parts' entries, mid rows and chunks, per side
+    Arena scratch, keep;
+    for (int b = 0; b < 2; ++b) {
+        scratch.add(&key[b], n);
+        scratch.add(&other[b], n);
+        scratch.add(&val[b], n);
+    }
+    scratch.add(&hist, scan_n);
+    scratch.add(&hscan, scan_n + 1);
+    scratch.add(&tmp, tmp_n);
+    scratch.add(&offs_dev, 6 * ((int64_t)B + 1));
+    for (int side = 0; side < 2; ++side) {
+        SideLayout &sd = c->side[side];
+        const int64_t nslots = (int64_t)B * (side == 0 ? I : J);
+        keep.add(&sd.ptr, nslots + 1);
+        keep.add(&sd.idx, n);
+        keep.add(&sd.val, n);
+        if (side == 0) keep.add(&sd.own, n);
+        keep.add(&sd.mid, std::min(n / (c->light_row + 1), nslots));
+        keep.add(&sd.heavy, max_chunks(n));
+    }
+    if (kept && (kept_bytes < keep.bytes || kept_bytes > 2 * keep.bytes)) {
+        dev_free(c, kept, st);
+        kept = nullptr;
+    }
+    void *scratch_mem = dev_alloc(c, scratch.bytes, st);
+    c->layout_mem = kept ? kept : dev_alloc(c, keep.bytes, st);
+    c->layout_bytes = kept ? kept_bytes : keep.bytes;
     auto cleanup = [&]() {
         cudaStreamSynchronize(st);   // the scratch is in use by work on st
-        for (void *p : scratch) dev_free(c, p, st);
+        dev_free(c, scratch_mem, st);
+        scratch_mem = nullptr;
     };
-#define PSGLD_ALLOC(ptr, cnt)                      \
-    do {                                           \
-        s = dmalloc(c, &(ptr), (cnt));             \
-        if (s != PSGLD_OK) { cleanup(); free_layout(c); return s; } \
-        scratch.push_back((void *)(ptr));          \
-    } while (0)
-    PSGLD_ALLOC(kA, n); PSGLD_ALLOC(kB, n); PSGLD_ALLOC(kt, n);
-    PSGLD_ALLOC(pA, n); PSGLD_ALLOC(pB, n); PSGLD_ALLOC(pt, n);
-    PSGLD_ALLOC(hist, scan_n); PSGLD_ALLOC(hscan, scan_n + 1); PSGLD_ALLOC(tmp, tmp_n);
-    int64_t *offs_dev = nullptr;
-    PSGLD_ALLOC(offs_dev, 3 * ((int64_t)B + 1));   // starts of the parts' entries, mid and heavy rows
-#undef PSGLD_ALLOC
+    auto give_up = [&](psgld_status s) {
+        cleanup();
+        free_layout(c);
+        return s;
+    };
+    if (!scratch_mem || !c->layout_mem)
+        return give_up(fail(c, PSGLD_ERR_OOM, "device allocation of " + std::to_string(scratch.bytes + keep.bytes) +
+                                                  " bytes for the layout failed"));
+    scratch.place(scratch_mem);
+    keep.place(c->layout_mem);
 
-    auto ck = [&](cudaError_t e, const char *what) -> psgld_status {
-        if (e != cudaSuccess) { cleanup(); free_layout(c); return cuda_fail(c, e, what); }
-        return PSGLD_OK;
-    };
-    if ((s = ck(cudaMemsetAsync(c->flag, 0, sizeof(int), st), "memset flag")) != PSGLD_OK) return s;
+    cudaError_t e = cudaMemsetAsync(c->flag, 0, sizeof(int), st);
     if (n > 0)
-        validate_and_key<<<grid_for(n, 256), 256, 0, st>>>(n, i_dev, j_dev, v_dev, I, J, B,
-                                                           c->prior.kind == PSGLD_PRIOR_EXPONENTIAL,
-                                                           bitsI, bitsJ, kA, kB, pA, pB, c->flag);
-    if ((s = ck(cudaGetLastError(), "validate_and_key")) != PSGLD_OK) return s;
+        validate_and_key<<<grid_for(n, 256), 256, 0, st>>>(n, i_dev, j_dev, v_dev, (uint32_t)I, (uint32_t)J, (uint32_t)B,
+                                                           c->prior.kind == PSGLD_PRIOR_EXPONENTIAL, key[0], c->flag);
+    if (e == cudaSuccess) e = cudaGetLastError();
     int hflag = 0;
-    if ((s = ck(cudaMemcpyAsync(&hflag, c->flag, sizeof(int), cudaMemcpyDeviceToHost, st), "flag d2h")) != PSGLD_OK) return s;
-    if ((s = ck(cudaStreamSynchronize(st), "sync")) != PSGLD_OK) return s;
-    if (hflag & 1) { cleanup(); free_layout(c); return fail(c, PSGLD_ERR_ARG, "entry index out of range"); }
-    if (hflag & 2) { cleanup(); free_layout(c); return fail(c, PSGLD_ERR_ARG, "entry value not finite, or negative in a non-negative model"); }
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&hflag, c->flag, sizeof(int), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return give_up(cuda_fail(c, e, "layout: entry checks"));
+    if (hflag & 1) return give_up(fail(c, PSGLD_ERR_ARG, "entry index out of range"));
+    if (hflag & 2) return give_up(fail(c, PSGLD_ERR_ARG, "entry value not finite, or negative in a non-negative model"));
 
+    const uint32_t *sorted = key[0];
     for (int side = 0; side < 2; ++side) {
         SideLayout &sd = c->side[side];
         const int64_t n_rows = side == 0 ? I : J;
         const int64_t nslots = (int64_t)B * n_rows;
-        uint64_t *k0 = side == 0 ? kA : kB;
-        uint32_t *v0 = side == 0 ? pA : pB;
-        uint64_t *k1 = kt;   // free again: the other side's finish_side ran first
-        uint32_t *v1 = pt;
         if (n > 0) {
-            s = radix_sort(c, k0, v0, k1, v1, n, side == 0 ? bitsA : bitsB, hist, hscan, tmp, st);
-            if (s != PSGLD_OK) { cleanup(); free_layout(c); return s; }
+            Entries in;
+            std::vector<Digit> ds;
+            if (side == 0) {
+                in = {key[0], reinterpret_cast<const uint32_t *>(j_dev), v_dev};
+                if (!(hflag & 8)) {
+                    ds = digits((uint32_t)I, bits_for((uint64_t)B), 0);
+                } else {
+                    ds = digits(1, bits_for((uint64_t)J), 1);
+                    for (const Digit &d : digits(1, bits_for((uint64_t)nslots), 0)) ds.push_back(d);
+                }
+            } else {
+                // the A side's sorted keys are in one of the two key arrays
+                uint32_t *kb = sorted == key[0] ? key[1] : key[0];
+                key_columns<<<grid_for(n, 256), 256, 0, st>>>(n, sorted, reinterpret_cast<const uint32_t *>(c->side[0].idx),
+                                                              (uint32_t)I, (uint32_t)J, kb, kb == key[0] ? other[0] : other[1]);
+                in = {kb, kb == key[0] ? other[0] : other[1], c->side[0].val};
+                ds = digits(1, bits_for((uint64_t)nslots), 0);
+            }
+            const psgld_status s = radix_sort(c, in, ds, n, key, other, val, reinterpret_cast<uint32_t *>(sd.idx), sd.val,
+                                              hist, hscan, tmp, &sorted, st);
+            if (s != PSGLD_OK) return give_up(s);
         }
-        s = dmalloc(c, &sd.ptr, nslots + 1);
-        if (s == PSGLD_OK) s = dmalloc(c, &sd.idx, n);
-        if (s == PSGLD_OK) s = dmalloc(c, &sd.val, n);
-        if (s == PSGLD_OK && side == 0) s = dmalloc(c, &sd.own, n);
-        if (s == PSGLD_OK) s = dmalloc(c, &sd.mid, std::min(n / (c->light_row + 1), nslots));
-        if (s == PSGLD_OK) s = dmalloc(c, &sd.heavy, max_chunks(n));
-        if (s != PSGLD_OK) { cleanup(); free_layout(c); return s; }
-        finish_side<<<grid_for(n + 1, 256), 256, 0, st>>>(n, k0, v0, side == 0 ? j_dev : i_dev, v_dev,
-                                                          side == 0 ? bitsJ : bitsI, nslots, n_rows,
-                                                          sd.idx, sd.val, sd.own, sd.ptr, c->flag);
-        if ((s = ck(cudaGetLastError(), "finish_side")) != PSGLD_OK) return s;
-        gather_starts<<<1, 128, 0, st>>>(reinterpret_cast<const uint32_t *>(sd.ptr), n_rows, B, offs_dev);
+        finish_side<<<grid_for(n + 1, 256), 256, 0, st>>>(n, sorted, reinterpret_cast<const uint32_t *>(sd.idx),
+                                                          (uint32_t)nslots, (uint32_t)n_rows, sd.own, sd.ptr, c->flag);
+        int64_t *offs = offs_dev + 3 * side * ((int64_t)B + 1);
+        gather_starts<<<1, 128, 0, st>>>(reinterpret_cast<const uint32_t *>(sd.ptr), n_rows, B, offs);
         for (int k = 0; k < 2; ++k) {
             count_rows<<<grid_for(nslots, 256), 256, 0, st>>>(sd.ptr, nslots, k, (uint32_t)c->light_row, hist);
-            s = exclusive_scan(c, hist, hscan, nslots, tmp, st);
-            if (s != PSGLD_OK) { cleanup(); free_layout(c); return s; }
+            const psgld_status s = exclusive_scan(c, hist, hscan, nslots, tmp, st);
+            if (s != PSGLD_OK) return give_up(s);
             list_rows<<<grid_for(nslots, 256), 256, 0, st>>>(hscan, nslots, n_rows, k == 0 ? sd.mid : nullptr,
                                                              k == 0 ? nullptr : sd.heavy);
-            gather_starts<<<1, 128, 0, st>>>(hscan, n_rows, B, offs_dev + (k + 1) * (B + 1));
+            gather_starts<<<1, 128, 0, st>>>(hscan, n_rows, B, offs + (k + 1) * (B + 1));
         }
-        if ((s = ck(cudaGetLastError(), "row lists")) != PSGLD_OK) return s;
-        std::vector<int64_t> h(3 * (size_t)(B + 1));
-        if ((s = ck(cudaMemcpyAsync(h.data(), offs_dev, sizeof(int64_t) * h.size(), cudaMemcpyDeviceToHost, st), "offsets d2h")) != PSGLD_OK) return s;
-        if ((s = ck(cudaStreamSynchronize(st), "sync")) != PSGLD_OK) return s;
+        e = cudaGetLastError();
+        if (e != cudaSuccess) return give_up(cuda_fail(c, e, "layout"));
+    }
+    std::vector<int64_t> h(6 * (size_t)(B + 1));
+    e = cudaMemcpyAsync(h.data(), offs_dev, sizeof(int64_t) * h.size(), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&hflag, c->flag, sizeof(int), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return give_up(cuda_fail(c, e, "layout: offsets"));
+    if (hflag & 4) return give_up(fail(c, PSGLD_ERR_ARG, "duplicate (i, j) entry"));
+    cleanup();
+
+    Arena chunk;
+    int64_t chunks[2];
+    for (int side = 0; side < 2; ++side) {
+        SideLayout &sd = c->side[side];
+        const int64_t *at = h.data() + 3 * side * (B + 1);
         if (side == 0) {
             c->part_n.resize(B);
-            for (int p = 0; p < B; ++p) c->part_n[p] = h[p + 1] - h[p];
+            for (int p = 0; p < B; ++p) c->part_n[p] = at[p + 1] - at[p];
         }
-        sd.mid_first.assign(h.begin() + (B + 1), h.begin() + 2 * (B + 1));
-        sd.heavy_first.assign(h.begin() + 2 * (B + 1), h.end());
-        int64_t chunks = 0;
-        for (int p = 0; p < B; ++p) chunks = std::max(chunks, sd.heavy_first[p + 1] - sd.heavy_first[p]);
-        if (chunks > 0) {
-            s = dmalloc(c, &sd.partial, chunks * c->ldk);
-            if (s == PSGLD_OK) s = dmalloc(c, &sd.arrived, chunks);
-            if (s != PSGLD_OK) { cleanup(); free_layout(c); return s; }
-            if ((s = ck(cudaMemsetAsync(sd.arrived, 0, sizeof(int) * (size_t)chunks, st), "memset chunks")) != PSGLD_OK)
-                return s;
+        sd.mid_first.assign(at + (B + 1), at + 2 * (B + 1));
+        sd.heavy_first.assign(at + 2 * (B + 1), at + 3 * (B + 1));
+        chunks[side] = 0;
+        for (int p = 0; p < B; ++p) chunks[side] = std::max(chunks[side], sd.heavy_first[p + 1] - sd.heavy_first[p]);
+        if (chunks[side] > 0) {
+            chunk.add(&sd.partial, chunks[side] * c->ldk);
+            chunk.add(&sd.arrived, chunks[side]);
         }
     }
-    if ((s = ck(cudaMemcpyAsync(&hflag, c->flag, sizeof(int), cudaMemcpyDeviceToHost, st), "flag d2h")) != PSGLD_OK) return s;
-    if ((s = ck(cudaStreamSynchronize(st), "sync")) != PSGLD_OK) return s;
-    cleanup();
-    if (hflag & 4) { free_layout(c); return fail(c, PSGLD_ERR_ARG, "duplicate (i, j) entry"); }
+    if (chunk.bytes > 0) {
+        c->chunk_mem = dev_alloc(c, chunk.bytes, st);
+        if (!c->chunk_mem) return give_up(fail(c, PSGLD_ERR_OOM, "device allocation failed"));
+        chunk.place(c->chunk_mem);
+        for (int side = 0; side < 2; ++side)
+            if (chunks[side] > 0) {
+                e = cudaMemsetAsync(c->side[side].arrived, 0, sizeof(int) * (size_t)chunks[side], st);
+                if (e != cudaSuccess) return give_up(cuda_fail(c, e, "memset"));
+            }
+    }
     c->N = n;
     c->has_data = true;
     return PSGLD_OK;
