@@ -351,6 +351,7 @@ psgld_status create_context(int64_t I, int64_t J, int32_t K, int32_t B, double t
     if (s == PSGLD_OK) c->red_host.assign(reduce_blocks(), 0.0);
     if (s == PSGLD_OK && cudaStreamSynchronize(zs) != cudaSuccess)
         s = fail(c, PSGLD_ERR_CUDA, "zero fill failed");
+    use_staging(1);
     if (s != PSGLD_OK) {
         psgld_destroy(c);
         cudaGetLastError();
@@ -690,23 +691,9 @@ psgld_status psgld_posterior_mean(psgld_ctx *c, double *Wm, double *Wv, double *
         psgld_status fs = check_kernel_flag(c);
         if (fs != PSGLD_OK) return fs;
     }
-    const int64_t ldk = c->ldk, K = c->K;
-    const double n = (double)c->n_samples;
-    for (int side = 0; side < 2; ++side) {
-        double *mean = side == 0 ? Wm : Hm, *var = side == 0 ? Wv : Hv;
-        if (!mean && !var) continue;
-        const int64_t rows = side == 0 ? c->I : c->J;
-        const Sums &S = side == 0 ? c->sW : c->sH;
-        std::vector<double> s((size_t)(rows * ldk)), s2((size_t)(rows * ldk));
-        PSGLD_CK(c, cudaMemcpy(s.data(), S.s, sizeof(double) * s.size(), cudaMemcpyDeviceToHost));
-        PSGLD_CK(c, cudaMemcpy(s2.data(), S.s2, sizeof(double) * s2.size(), cudaMemcpyDeviceToHost));
-        for (int64_t r = 0; r < rows; ++r)
-            for (int64_t k = 0; k < K; ++k) {
-                const double m = n > 0 ? s[r * ldk + k] / n : 0.0;
-                if (mean) mean[r * K + k] = m;
-                if (var) var[r * K + k] = n > 0 ? s2[r * ldk + k] / n - m * m : 0.0;
-            }
-    }
+    double *const out[2][2] = {{Wm, Wv}, {Hm, Hv}};
+    const psgld_status s = read_moments(c, out);
+    if (s != PSGLD_OK) return s;
     if (n_samples) *n_samples = c->n_samples;
     return PSGLD_OK;
 }
@@ -1155,6 +1142,7 @@ void psgld_destroy(psgld_ctx *c)
     dev_free(c, c->eps_tab);
     if (c->capture_stream) cudaStreamDestroy(c->capture_stream);
     delete c;
+    use_staging(-1);
 }
 
 }  // extern "C"

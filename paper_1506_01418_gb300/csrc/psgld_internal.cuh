@@ -312,6 +312,13 @@ psgld_status launch_eps_table(psgld_ctx *c, cudaStream_t st);
 psgld_status reduce_loglik_rmse(psgld_ctx *c, int mode, int use_mean,
                                 cudaStream_t st, double *out);
 
+// ---- read-back (psgld_readout.cu) -------------------------------------------
+// Posterior means and variances, out[side][0 / 1], rows x K each (null: not
+// wanted), complete on return; the context's work must be done.
+psgld_status read_moments(psgld_ctx *c, double *const (&out)[2][2]);
+// A context more (1) or less (-1): the staging memory lives while any does.
+void use_staging(int by);
+
 // ---- scans and sorts (psgld_layout.cu) ------------------------------------
 int bits_for(uint64_t n_values);
 
