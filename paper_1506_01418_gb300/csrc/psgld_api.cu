@@ -847,6 +847,10 @@ psgld_status psgld_batch_sweep(psgld_ctx *const *ctxs, int32_t n, int32_t n_swee
         gbeg.push_back((int)order.size());
         for (int i = 0; i < n; ++i)
             if (dense_batch_key(ctxs[i]) == key) order.push_back(i);
+        // the longest items first: a part's launch ends with its last one
+        std::stable_sort(order.begin() + gbeg.back(), order.end(), [&](int a, int b) {
+            return dense_batch_length(ctxs[a]) > dense_batch_length(ctxs[b]);
+        });
     }
     gbeg.push_back(n);
     const int ng = (int)keys.size();
@@ -1105,7 +1109,7 @@ int64_t psgld_estimate_device_bytes(int64_t I, int64_t J, int32_t K, int32_t B, 
     int dev = 0, sms = 152;
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const bool share = two_sided_share(-1, maxI, B, (int)mt, (int)nt, sms) != 0;
-    bytes += (int64_t)B * B * mt * nj * 8192 * vs;                 // V tiles
+    bytes += (int64_t)B * B * mt * nj * 64 * (share ? 128 : rc_tile_rows(maxI)) * vs;   // V tiles
     if (!share) bytes += (int64_t)B * B * nt * ni * 8192 * vs;     // ... other orientation
     bytes += (int64_t)B * 2 * (mt + nt) * 64 * KP * 2;              // BF16 factor shadows
     if (share) bytes += (int64_t)B * mt * 4 * cdiv(maxJ, 256) * 8192 * 2;   // one part's E

@@ -586,7 +586,7 @@ dense_grad_batch_kernel(const unsigned char *__restrict__ tab, size_t stride, co
 // kernel), and V cut into 128 x 64 tiles per block, once per orientation, in
 // the order the epilogue reads them (4-column FP32 or 8-column BF16 chunks,
 // one 16-byte chunk per owned row, so a warp reads 512 contiguous bytes).
-// Every tile is one bulk copy.  Items are assigned to CTAs round robin.
+// Every tile is one bulk copy.  Items are assigned to CTAs in rounds.
 //
 // One persistent CTA per SM, 10 warps:
 //   warp 0               producer: the owned tile once per item, then per
@@ -626,9 +626,10 @@ struct Side {
     const uint16_t *walk_sh;    // ... of the walked factor
     const unsigned char *Vt;    // V tiles in this orientation
     float *G;                   // G rows of the owned factor
-    int64_t n_own, n_walk;      // I or J
+    uint32_t n_own, n_walk;     // I or J
     int own_tiles;              // 128-row tile slots per owned piece (items, V tiles)
     int walk_tiles;             // 64-row V tile slots per walked piece
+    int ht;                     // rows of a V tile (128, or fewer when pieces are shorter)
     int own_sh64, walk_sh64;    // 64-row shadow tiles per owned / walked piece
 };
 
@@ -767,24 +768,27 @@ struct Item {
     int64_t own_start;
 };
 
+// 32-bit arithmetic throughout: B I and B J are below 2^31 (checked at
+// create), and an item of a short chain is over in a few microseconds.
 __device__ __forceinline__ bool decode(const Params &P, int it, Item &x)
 {
-    const int B = P.B;
-    int side = 0, k = it;
-    if (k >= P.items_a) { side = 1; k -= P.items_a; }
+    const uint32_t B = (uint32_t)P.B;
+    int side = 0;
+    uint32_t k = (uint32_t)it;
+    if (it >= P.items_a) { side = 1; k -= (uint32_t)P.items_a; }
     const Side &Sd = P.side[side];
-    const int b = k / Sd.own_tiles, ot = k % Sd.own_tiles;
-    const int cpiece = (b + P.part) % B;
+    const uint32_t b = k / (uint32_t)Sd.own_tiles, ot = k - b * (uint32_t)Sd.own_tiles;
+    const uint32_t to = b + (uint32_t)P.part, cpiece = to < B ? to : to - B;
+    const uint32_t own = side == 0 ? b : cpiece, walk = side == 0 ? cpiece : b;
     x.side = side;
-    x.own_piece = side == 0 ? b : cpiece;
-    x.walk_piece = side == 0 ? cpiece : b;
-    x.ot = ot;
-    x.own_start = ((int64_t)x.own_piece * Sd.n_own) / B;
-    const int64_t own_rows = ((int64_t)(x.own_piece + 1) * Sd.n_own) / B - x.own_start;
-    const int64_t walk_rows = ((int64_t)(x.walk_piece + 1) * Sd.n_walk) / B -
-                              ((int64_t)x.walk_piece * Sd.n_walk) / B;
-    const int64_t left = own_rows - (int64_t)ot * kOwn;
-    x.own_rows_in_tile = (int)(left < kOwn ? left : kOwn);
+    x.own_piece = (int)own;
+    x.walk_piece = (int)walk;
+    x.ot = (int)ot;
+    const uint32_t start = own * Sd.n_own / B;
+    x.own_start = start;
+    const int left = (int)((own + 1) * Sd.n_own / B - start) - (int)ot * kOwn;
+    x.own_rows_in_tile = left < kOwn ? left : kOwn;
+    const uint32_t walk_rows = (walk + 1) * Sd.n_walk / B - walk * Sd.n_walk / B;
     x.nj = (int)((walk_rows + kBN - 1) / kBN);
     return left > 0;
 }
@@ -804,30 +808,52 @@ __device__ __forceinline__ float tweedie_pm(float p, float phi_inv, float mu_min
 }
 
 // Where the items' parameters come from: one context (the kernel parameter)
-// or, batched, a table of contexts in global memory whose items follow one
-// another (context i owns items [item_start[i], item_start[i + 1]); slots
-// `stride` bytes apart).
+// or, batched, a table of contexts in global memory (slots `stride` bytes
+// apart) with two prefixes of their items: rows items of every context first,
+// then columns items (a context's rows items walk its long side).
 struct Src {
     const unsigned char *tab;
-    const int *item_start;
+    const int *rows_start, *cols_start;
     int n;
     size_t stride;
 };
 
+// Items in rounds of the grid, every other round backwards: of items that
+// come longest first, the block with the longest of one round takes the
+// shortest of the next.
+__device__ __forceinline__ int round_item(int round)
+{
+    const int g = (int)gridDim.x, k = (int)blockIdx.x;
+    return round * g + (round & 1 ? g - 1 - k : k);
+}
+
+// The context of a warp's next item, its items of one kind ascending.
+struct Place {
+    int kind = 0, ctx = 0;
+};
+
+// A whole warp looks among the next 32 contexts after the last item's at a
+// time.
 template <bool BATCH>
-__device__ __forceinline__ const Params &ctx_of(const Params &P0, const Src &src, int it, int &local)
+__device__ __forceinline__ const Params &ctx_of(const Params &P0, const Src &src, int it, int &local, Place &at)
 {
     if constexpr (!BATCH) {
         local = it;
         return P0;
     } else {
-        int lo = 0, hi = src.n - 1;          // last i with item_start[i] <= it
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (__ldg(src.item_start + mid) <= it) lo = mid; else hi = mid - 1;
+        const int rows = __ldg(src.rows_start + src.n);
+        if (at.kind == 0 && it >= rows) at = Place{1, 0};
+        const int *start = at.kind ? src.cols_start : src.rows_start;
+        if (at.kind) it -= rows;
+        for (;;) {
+            const int k = at.ctx + 1 + (int)(threadIdx.x & 31);
+            const int past = __popc(__ballot_sync(0xffffffffu, k < src.n && __ldg(start + k) <= it));
+            at.ctx += past;
+            if (past < 32) break;
         }
-        local = it - __ldg(src.item_start + lo);
-        return *reinterpret_cast<const Params *>(src.tab + (size_t)lo * src.stride);
+        const Params &P = *reinterpret_cast<const Params *>(src.tab + (size_t)at.ctx * src.stride);
+        local = it - __ldg(start + at.ctx) + (at.kind ? P.items_a : 0);
+        return P;
     }
 }
 
@@ -884,10 +910,12 @@ __device__ __forceinline__ void chain_body(const Params &P0, const Src src, int 
         {
             const uint32_t ld = lane == 0;
             uint32_t ic = 0;
+            Place place;
             Ring rb, rv;
-            for (int it = blockIdx.x; it < total_items; it += gridDim.x) {
+            for (int round = 0, it; round * (int)gridDim.x < total_items; ++round) {
+                if ((it = round_item(round)) >= total_items) continue;
                 int lit;
-                const Params &P = ctx_of<BATCH>(P0, src, it, lit);
+                const Params &P = ctx_of<BATCH>(P0, src, it, lit, place);
                 Item x;
                 if (!decode(P, lit, x)) continue;
                 const Side &Sd = P.side[x.side];
@@ -902,9 +930,10 @@ __device__ __forceinline__ void chain_body(const Params &P0, const Src src, int 
                         bulk_g2s_if(ld, sA + a * 16384 + 8192, t0 + 64 * KP + a * 4096, 8192, &S->a_full);
                     }
                 }
+                const uint32_t vb = (uint32_t)Sd.ht * kBN * sizeof(VT);   // the V tile as it is stored
                 const unsigned char *vbase =
                     Sd.Vt + ((((int64_t)x.own_piece * P.B + x.walk_piece) * Sd.own_tiles + x.ot) *
-                             Sd.walk_tiles) * (int64_t)v_bytes;
+                             Sd.walk_tiles) * (int64_t)vb;
                 for (int j = 0; j < x.nj; ++j) {
                     const uint32_t st = rb.slot, sv = rv.slot;
                     if (!wait32(S, &S->empty[st], rb.phase ^ 1)) goto done0;
@@ -913,8 +942,8 @@ __device__ __forceinline__ void chain_body(const Params &P0, const Src src, int 
                                 Sd.walk_sh + ((int64_t)x.walk_piece * Sd.walk_sh64 + j) * kBN * KP,
                                 b_bytes, &S->full[st]);
                     if (!wait32(S, &S->vempty[sv], rv.phase ^ 1)) goto done0;
-                    expect_tx_if(ld, &S->vfull[sv], v_bytes);
-                    bulk_g2s_if(ld, sV + (size_t)sv * v_bytes, vbase + (int64_t)j * v_bytes, v_bytes, &S->vfull[sv]);
+                    expect_tx_if(ld, &S->vfull[sv], vb);
+                    bulk_g2s_if(ld, sV + (size_t)sv * v_bytes, vbase + (int64_t)j * vb, vb, &S->vfull[sv]);
                     rb.next(NS);
                     rv.next(NV);
                 }
@@ -930,6 +959,7 @@ __device__ __forceinline__ void chain_body(const Params &P0, const Src src, int 
         {
             const uint32_t ld = lane == 0;
             uint32_t tc = 0, ic = 0;
+            Place place;
             Ring r1, r2;     // walked-tile slots of GEMM1 (tile tc) and GEMM2 (tile tc - 1)
             const uint32_t id1 = idesc_bf16(kOwn, kBN);
             const uint32_t id2 = idesc_bf16(kOwn, KP, 0, 1);
@@ -938,9 +968,10 @@ __device__ __forceinline__ void chain_body(const Params &P0, const Src src, int 
             // next atom of the owned tile starts 128 rows x 128 B further
             const uint32_t aA = saddr(sA);
             const uint32_t tA = tmem + (kTmemCols - (uint32_t)KP / 2);   // owned tile in TMEM
-            for (int it = blockIdx.x; it < total_items; it += gridDim.x) {
+            for (int round = 0, it; round * (int)gridDim.x < total_items; ++round) {
+                if ((it = round_item(round)) >= total_items) continue;
                 int lit;
-                const Params &P = ctx_of<BATCH>(P0, src, it, lit);
+                const Params &P = ctx_of<BATCH>(P0, src, it, lit, place);
                 Item x;
                 if (!decode(P, lit, x)) continue;
                 if (!wait32(S, &S->a_full, ic & 1)) goto done1;
@@ -1011,14 +1042,20 @@ __device__ __forceinline__ void chain_body(const Params &P0, const Src src, int 
         const int c = 32 * hc;
         const uint32_t lane_base = (uint32_t)(32 * q) << 16;
         uint32_t tc = 0, ic = 0;
+        Place place;
         Ring rv;
-        for (int it = blockIdx.x; it < total_items; it += gridDim.x) {
+        for (int round = 0, it; round * (int)gridDim.x < total_items; ++round) {
+            if ((it = round_item(round)) >= total_items) continue;
             int lit;
-            const Params &P = ctx_of<BATCH>(P0, src, it, lit);
+            const Params &P = ctx_of<BATCH>(P0, src, it, lit, place);
             Item x;
             if (!decode(P, lit, x)) continue;
             const Side &Sd = P.side[x.side];
             const float pp = P.p, phi_inv = P.phi_inv, mu_min = P.mu_min;
+            const int ht = Sd.ht;
+            // a warp whose rows are all past the piece forms no E: whatever E
+            // holds there only reaches G rows that nobody reads
+            const bool work = 32 * q < x.own_rows_in_tile;
             for (int j = 0; j < x.nj; ++j, ++tc, rv.next(NV)) {
                 const int b = (int)(tc & 1);
                 const uint32_t sv = rv.slot;
@@ -1027,45 +1064,47 @@ __device__ __forceinline__ void chain_body(const Params &P0, const Src src, int 
                 if (!wait32(S, &S->mu_full[b], ph)) goto done2;
                 if (!wait32(S, &S->e_empty[b], ph ^ 1)) goto done2;
                 fence_after();
-                const unsigned char *vt = sV + (size_t)sv * v_bytes;
-                unsigned char *eb = sE + b * e_bytes;
-                float mu[32];
-                tmem_ld32(tmem + lane_base + (uint32_t)(b * kBN + c), mu);
-                float v[32];
-                if constexpr (sizeof(VT) == 4) {
+                if (work) {
+                    const unsigned char *vt = sV + (size_t)sv * v_bytes;
+                    unsigned char *eb = sE + b * e_bytes;
+                    float mu[32];
+                    tmem_ld32(tmem + lane_base + (uint32_t)(b * kBN + c), mu);
+                    float v[32];
+                    if constexpr (sizeof(VT) == 4) {
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        const float4 w = *reinterpret_cast<const float4 *>(
-                            vt + ((size_t)((c >> 2) + i) * kOwn + rho) * 16);
-                        v[4 * i] = w.x; v[4 * i + 1] = w.y; v[4 * i + 2] = w.z; v[4 * i + 3] = w.w;
-                    }
-                } else {
+                        for (int i = 0; i < 8; ++i) {
+                            const float4 w = *reinterpret_cast<const float4 *>(
+                                vt + ((size_t)((c >> 2) + i) * ht + rho) * 16);
+                            v[4 * i] = w.x; v[4 * i + 1] = w.y; v[4 * i + 2] = w.z; v[4 * i + 3] = w.w;
+                        }
+                    } else {
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const uint4 w = *reinterpret_cast<const uint4 *>(
-                            vt + ((size_t)((c >> 3) + i) * kOwn + rho) * 16);
-                        const uint32_t u[4] = {w.x, w.y, w.z, w.w};
+                        for (int i = 0; i < 4; ++i) {
+                            const uint4 w = *reinterpret_cast<const uint4 *>(
+                                vt + ((size_t)((c >> 3) + i) * ht + rho) * 16);
+                            const uint32_t u[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
-                        for (int h = 0; h < 4; ++h) {
-                            v[8 * i + 2 * h] = __uint_as_float(u[h] << 16);
-                            v[8 * i + 2 * h + 1] = __uint_as_float(u[h] & 0xffff0000u);
+                            for (int h = 0; h < 4; ++h) {
+                                v[8 * i + 2 * h] = __uint_as_float(u[h] << 16);
+                                v[8 * i + 2 * h + 1] = __uint_as_float(u[h] & 0xffff0000u);
+                            }
                         }
                     }
-                }
-                uint32_t pk[16];
+                    uint32_t pk[16];
 #pragma unroll
-                for (int h = 0; h < 16; ++h) {
-                    const float e0 = tweedie_pm<PM>(pp, phi_inv, mu_min, v[2 * h], mu[2 * h]);
-                    const float e1 = tweedie_pm<PM>(pp, phi_inv, mu_min, v[2 * h + 1], mu[2 * h + 1]);
-                    __nv_bfloat162 t2 = __floats2bfloat162_rn(e0, e1);
-                    pk[h] = *reinterpret_cast<uint32_t *>(&t2);
-                }
-                // E (owned row rho, walked columns c..c+31): row rho of the
-                // 128-byte-swizzled atom column, chunk (c/8 + g) ^ (rho % 8)
+                    for (int h = 0; h < 16; ++h) {
+                        const float e0 = tweedie_pm<PM>(pp, phi_inv, mu_min, v[2 * h], mu[2 * h]);
+                        const float e1 = tweedie_pm<PM>(pp, phi_inv, mu_min, v[2 * h + 1], mu[2 * h + 1]);
+                        __nv_bfloat162 t2 = __floats2bfloat162_rn(e0, e1);
+                        pk[h] = *reinterpret_cast<uint32_t *>(&t2);
+                    }
+                    // E (owned row rho, walked columns c..c+31): row rho of the
+                    // 128-byte-swizzled atom column, chunk (c/8 + g) ^ (rho % 8)
 #pragma unroll
-                for (int g = 0; g < 4; ++g)
-                    *reinterpret_cast<uint4 *>(eb + rho * 128 + ((((c >> 3) + g) ^ (rho & 7)) << 4)) =
-                        make_uint4(pk[4 * g], pk[4 * g + 1], pk[4 * g + 2], pk[4 * g + 3]);
+                    for (int g = 0; g < 4; ++g)
+                        *reinterpret_cast<uint4 *>(eb + rho * 128 + ((((c >> 3) + g) ^ (rho & 7)) << 4)) =
+                            make_uint4(pk[4 * g], pk[4 * g + 1], pk[4 * g + 2], pk[4 * g + 3]);
+                }
                 fence_async_smem();
                 fence_before();
                 __syncwarp();
@@ -1078,7 +1117,7 @@ __device__ __forceinline__ void chain_body(const Params &P0, const Src src, int 
             // the item's G rows: this warp's lane quarter, every other 32-column chunk
             if (!wait32(S, &S->g_full, ic & 1)) goto done2;
             fence_after();
-            {
+            if (work) {
                 const bool rv = rho < x.own_rows_in_tile;
                 float *dst = Sd.G + (x.own_start + (int64_t)x.ot * kOwn + rho) * P.ldk;
                 for (int cc = 32 * hc; cc < KP; cc += 64) {
@@ -1121,16 +1160,17 @@ __device__ __forceinline__ void chain_body(const Params &P0, const Src src, int 
 template <typename VT, int PM>
 __global__ void __launch_bounds__(kThreads, 1) chain_kernel(const __grid_constant__ Params P)
 {
-    chain_body<VT, PM, false>(P, Src{nullptr, nullptr, 1, 0}, P.items, false);
+    chain_body<VT, PM, false>(P, Src{nullptr, nullptr, nullptr, 1, 0}, P.items, false);
 }
 
 // Many contexts of one K width, V type and power in one persistent launch.
 template <typename VT, int PM>
 __global__ void __launch_bounds__(kThreads, 1)
-chain_batch_kernel(const unsigned char *tab, size_t stride, const int *item_start, int n, int late)
+chain_batch_kernel(const unsigned char *tab, size_t stride, const int *rows_start, const int *cols_start, int n,
+                   int late)
 {
-    chain_body<VT, PM, true>(*reinterpret_cast<const Params *>(tab), Src{tab, item_start, n, stride},
-                             __ldg(item_start + n), late != 0);
+    chain_body<VT, PM, true>(*reinterpret_cast<const Params *>(tab), Src{tab, rows_start, cols_start, n, stride},
+                             __ldg(rows_start + n) + __ldg(cols_start + n), late != 0);
 }
 
 }  // namespace two_sided_rc
@@ -2170,10 +2210,10 @@ __device__ __forceinline__ int64_t piece_start_d(int64_t r, int64_t n, int B) { 
 __device__ __forceinline__ int64_t piece_of_d(int64_t x, int64_t n, int B) { return ((x + 1) * B - 1) / n; }
 
 // V (I x J, FP32, row-major) into the tiles of one orientation (side 0: owned
-// = rows of V, side 1: owned = columns); padding stays zero.
+// = rows of V, side 1: owned = columns), of ht owned rows; padding stays zero.
 template <typename VT>
 __global__ void build_vtiles_kernel(const float *__restrict__ V, int64_t I, int64_t J, int B, int side,
-                                    int own_tiles, int walk_tiles, VT *__restrict__ out)
+                                    int own_tiles, int walk_tiles, int ht, VT *__restrict__ out)
 {
     const int64_t n_own = side == 0 ? I : J, n_walk = side == 0 ? J : I;
     for (int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; a < I * J;
@@ -2186,9 +2226,9 @@ __global__ void build_vtiles_kernel(const float *__restrict__ V, int64_t I, int6
         const int rho = (int)(orow & 127), kap = (int)(wrow & 63);
         int64_t e;
         if constexpr (sizeof(VT) == 4)
-            e = tile * 8192 + ((int64_t)(kap >> 2) * 128 + rho) * 4 + (kap & 3);
+            e = (tile * 16 + (kap >> 2)) * 4 * ht + rho * 4 + (kap & 3);
         else
-            e = tile * 8192 + ((int64_t)(kap >> 3) * 128 + rho) * 8 + (kap & 7);
+            e = (tile * 8 + (kap >> 3)) * 8 * ht + rho * 8 + (kap & 7);
         if constexpr (sizeof(VT) == 4)
             out[e] = V[a];
         else
@@ -2220,7 +2260,7 @@ ChainRcFn pick_chain_rc(bool vb, int pm)
     return f[vb ? 1 : 0][pm];
 }
 
-using ChainRcBatchFn = void (*)(const unsigned char *, size_t, const int *, int, int);
+using ChainRcBatchFn = void (*)(const unsigned char *, size_t, const int *, const int *, int, int);
 
 ChainRcBatchFn pick_chain_batch_rc(bool vb, int pm)
 {
@@ -2382,7 +2422,8 @@ psgld_status prepare_dense(psgld_ctx *c, cudaStream_t st)
     PSGLD_CK(c, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device));
     c->share_e = two_sided_share(c->opt.dense_share_e, maxI, c->B, c->mt_max, c->nt_max, sms);
     const int64_t B = c->B;
-    const int64_t nA = B * B * c->mt_max * c->nj_max * 8192;
+    c->vt_rows = c->share_e ? 128 : rc_tile_rows(maxI);
+    const int64_t nA = B * B * c->mt_max * c->nj_max * 64 * c->vt_rows;
     const int64_t nB = c->share_e ? 0 : B * B * c->nt_max * c->ni_max * 8192;   // V tiles, other orientation
     const int64_t nW = B * 2 * c->mt_max * 64 * c->KP, nH = B * 2 * c->nt_max * 64 * c->KP;
     const int64_t nE = c->share_e ? B * c->mt_max * 4 * c->nt2_max * 8192 : 0;   // one part's E tiles
@@ -2428,13 +2469,14 @@ psgld_status build_dense_tiles(psgld_ctx *c, cudaStream_t st)
     for (int side = 0; side < (c->share_e ? 1 : 2); ++side) {
         const int own_tiles = side == 0 ? c->mt_max : c->nt_max;
         const int walk_tiles = side == 0 ? c->nj_max : c->ni_max;
+        const int ht = side == 0 ? c->vt_rows : 128;
         void *out = side == 0 ? c->VA : c->VB;
         if (c->v_bf16)
             build_vtiles_kernel<__nv_bfloat16><<<grid, 256, 0, st>>>(c->Vd, c->I, c->J, c->B, side, own_tiles,
-                                                                      walk_tiles, (__nv_bfloat16 *)out);
+                                                                      walk_tiles, ht, (__nv_bfloat16 *)out);
         else
             build_vtiles_kernel<float><<<grid, 256, 0, st>>>(c->Vd, c->I, c->J, c->B, side, own_tiles,
-                                                              walk_tiles, (float *)out);
+                                                              walk_tiles, ht, (float *)out);
         PSGLD_CK(c, cudaGetLastError());
     }
     return PSGLD_OK;
@@ -2465,6 +2507,8 @@ psgld_status build_dense_shadows(psgld_ctx *c, cudaStream_t st)
 // part's items fill more than one wave of CTAs; short pieces or a single
 // wave favour columns items that form their own mu, all items at once.
 // The option overrides the rule (-1 = the rule).
+int rc_tile_rows(int64_t max_rows) { return max_rows >= 128 ? 128 : 32 * (int)((max_rows + 31) / 32); }
+
 int two_sided_share(int opt, int64_t max_rows, int B, int mt, int nt, int sms)
 {
     if (opt >= 0) return opt;
@@ -2519,6 +2563,7 @@ static void fill_rc(const psgld_ctx *c, int part, two_sided_rc::Params &P)
     A.own_sh = c->Wsh; A.walk_sh = c->Hsh; A.Vt = (const unsigned char *)c->VA; A.G = c->G;
     A.n_own = I; A.n_walk = J; A.own_tiles = c->mt_max; A.walk_tiles = c->nj_max;
     A.own_sh64 = 2 * c->mt_max; A.walk_sh64 = 2 * c->nt_max;
+    A.ht = c->vt_rows; Bs.ht = 128;
     Bs.own_sh = c->Hsh; Bs.walk_sh = c->Wsh; Bs.Vt = (const unsigned char *)c->VB; Bs.G = c->G + I * c->ldk;
     Bs.n_own = J; Bs.n_walk = I; Bs.own_tiles = c->nt_max; Bs.walk_tiles = c->ni_max;
     Bs.own_sh64 = 2 * c->nt_max; Bs.walk_sh64 = 2 * c->mt_max;
@@ -2606,6 +2651,8 @@ psgld_status launch_dense_grad(psgld_ctx *c, int part, cudaStream_t st)
 // Batch keys: single-pass 2 KP + fp8 (< 4096); two-sided 4096 + 8 KP +
 // 4 v_bf16 + power mode (the chain kernel's template arguments), plus 8192
 // for the shared-E kernel.
+int dense_batch_length(const psgld_ctx *c) { return c->dense_kind == 2 ? std::max(c->ni_max, c->nj_max) : 0; }
+
 int dense_batch_key(const psgld_ctx *c)
 {
     if (c->dense_kind == 1) return 2 * dense_kp(c->K) + c->dense_fp8;
@@ -2628,7 +2675,7 @@ int fill_dense_param(const psgld_ctx *c, int part, void *dst, int *first_items)
         two_sided_rc::Params P;
         fill_rc(c, part, P);
         std::memcpy(dst, &P, sizeof P);
-        *first_items = P.items;
+        *first_items = P.items_a;   // the rows items, then the columns items
         return P.items;
     }
     if (c->dense_kind == 2) {
@@ -2653,7 +2700,7 @@ psgld_status launch_dense_batch(psgld_ctx *c0, int key, const void *params, cons
     const size_t stride = dense_param_bytes();
     if (key >= 4096 && key < 8192) {
         // two-sided contexts whose items form their own mu: one persistent
-        // launch over all their items, round robin (cta_start: their prefix)
+        // launch over all their items (cta_start: their two prefixes)
         const int KP = (key - 4096) / 8;
         const bool vb = ((key >> 2) & 1) != 0;
         const int pm = key & 3;
@@ -2669,7 +2716,7 @@ psgld_status launch_dense_batch(psgld_ctx *c0, int key, const void *params, cons
         if (c0->opt.batch_ctas > 0) grid = std::min(grid, (int)c0->opt.batch_ctas);
         if (grid > 0)
             PSGLD_CK(c0, launch_early(early, fn, (unsigned)grid, two_sided_rc::kThreads, smem, st, tab, stride, cta_start,
-                                      n, early && late ? 1 : 0));
+                                      cta_start + n + 1, n, early && late ? 1 : 0));
         return PSGLD_OK;
     }
     if (key >= 8192) {

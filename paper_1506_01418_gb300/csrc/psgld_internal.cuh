@@ -115,6 +115,7 @@ struct psgld_ctx {
     int mt_max = 0, nt_max = 0;      // 128-row tiles per row piece / column piece
     int nt2_max = 0;                 // 256-row column tiles per column piece (columns items)
     int ni_max = 0, nj_max = 0;      // 64-row tiles per row piece / column piece
+    int vt_rows = 128;               // rows of VA's tiles
 
     // factors
     float *W[2] = {nullptr, nullptr};
@@ -259,6 +260,10 @@ psgld_status prepare_dense(psgld_ctx *c, cudaStream_t st);
 // Whether the two-sided kernel's columns items take E from the rows items
 // (opt >= 0: as given; -1: long row pieces and more than one wave of items).
 int two_sided_share(int opt, int64_t max_rows, int B, int mt, int nt, int sms);
+// Rows of V's tiles for row pieces of at most max_rows (two-sided kernel whose
+// items form their own mu): a tile shorter than the tensor core's 128 rows is
+// read and stored as such.
+int rc_tile_rows(int64_t max_rows);
 // V tiles of the two-sided kernel from c->Vd (no-op for the single-pass one).
 psgld_status build_dense_tiles(psgld_ctx *c, cudaStream_t st);
 // BF16 shadows of the current factors (two-sided kernel with factors set).
@@ -282,6 +287,9 @@ psgld_status launch_dense_grad(psgld_ctx *c, int part, cudaStream_t st);
 // cta_start holds two prefix arrays of n + 1 entries: rows items, then
 // columns items.
 int dense_batch_key(const psgld_ctx *c);
+// Tiles an item of the context walks at most: contexts of a launch come in
+// descending order of it.
+int dense_batch_length(const psgld_ctx *c);
 size_t dense_param_bytes();
 int fill_dense_param(const psgld_ctx *c, int part, void *dst, int *first_items);
 // late (not the part's first gradient launch): the launch waits for the one
