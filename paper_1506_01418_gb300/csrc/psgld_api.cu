@@ -1091,8 +1091,8 @@ int64_t psgld_estimate_device_bytes(int64_t I, int64_t J, int32_t K, int32_t B, 
         // the lists of the rows with many entries and their chunks' sums
         for (int side = 0; side < 2; ++side) {
             const int64_t n_rows = side == 0 ? I : J;
-            bytes += (B * n_rows + 1) * 4 + nnz * (side == 0 ? 12 : 8) + 4 * std::min(nnz / (light_row_for(I + J) + 1), B * n_rows) +
-                     8 * max_chunks(nnz) + (4 * ldk + 4) * std::min(max_chunks(nnz), max_chunks(cdiv(nnz, B)) + n_rows);
+            bytes += (B * n_rows + 1) * 4 + nnz * (side == 0 ? 12 : 8) +
+                     16 * (std::min(nnz / (light_row_for(I + J) + 1), B * n_rows) + max_chunks(nnz)) + (4 * ldk + 4) * std::min(max_chunks(nnz), max_chunks(cdiv(nnz, B)) + n_rows);
         }
         return bytes;
     }

@@ -45,10 +45,10 @@ struct SideLayout {
     float *val = nullptr;      // value of each entry
     int32_t *own = nullptr;    // A side: own row of each entry (log-likelihood, RMSE)
     // per part, the rows with more than light_row and at most kMidRow entries
-    // in it, ascending, and the chunks (row, number) of kChunk entries of the
-    // rows with more; part s: [first[s], first[s + 1])
-    int32_t *mid = nullptr;
-    int2 *heavy = nullptr;
+    // in it (row, first entry, entries, 0), ascending, and the chunks of
+    // kChunk entries of the rows with more (row, first entry, entries, number
+    // of the chunk); part s: [first[s], first[s + 1])
+    int4 *mid = nullptr, *heavy = nullptr;
     std::vector<int64_t> mid_first, heavy_first;
     float *partial = nullptr;  // ldk sums per chunk of the part with the most chunks
     int *arrived = nullptr;    // per chunk: of a row's first one, how many are done

@@ -317,15 +317,16 @@ __global__ void count_rows(const int32_t *__restrict__ ptr, int64_t nslots, int 
 
 // The mid rows, or the heavy rows' chunks, in slot order (pos: exclusive
 // scan of count_rows).
-__global__ void list_rows(const uint32_t *__restrict__ pos, int64_t nslots, int64_t n_rows,
-                          int32_t *__restrict__ mid, int2 *__restrict__ heavy)
+__global__ void list_rows(const uint32_t *__restrict__ pos, const int32_t *__restrict__ ptr, int64_t nslots,
+                          uint32_t n_rows, int4 *__restrict__ list)
 {
     for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < nslots;
          s += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t a = pos[s], b = pos[s + 1];
-        if (mid && b > a) mid[a] = (int32_t)(s % n_rows);
-        if (heavy)
-            for (uint32_t k = a; k < b; ++k) heavy[k] = make_int2((int)(s % n_rows), (int)(k - a));
+        if (b > a) {
+            const int row = (int)((uint32_t)s % n_rows), first = ptr[s], n = ptr[s + 1] - first;
+            for (uint32_t k = a; k < b; ++k) list[k] = make_int4(row, first, n, (int)(k - a));
+        }
     }
 }
 
@@ -550,8 +551,8 @@ psgld_status build_layout(psgld_ctx *c, int64_t nnz, const int32_t *i_dev, const
             count_rows<<<grid_for(nslots, 256), 256, 0, st>>>(sd.ptr, nslots, k, (uint32_t)c->light_row, hist);
             const psgld_status s = exclusive_scan(c, hist, hscan, nslots, tmp, st);
             if (s != PSGLD_OK) return give_up(s);
-            list_rows<<<grid_for(nslots, 256), 256, 0, st>>>(hscan, nslots, n_rows, k == 0 ? sd.mid : nullptr,
-                                                             k == 0 ? nullptr : sd.heavy);
+            list_rows<<<grid_for(nslots, 256), 256, 0, st>>>(hscan, sd.ptr, nslots, (uint32_t)n_rows,
+                                                             k == 0 ? sd.mid : sd.heavy);
             gather_starts<<<1, 128, 0, st>>>(hscan, n_rows, B, offs + (k + 1) * (B + 1));
         }
         e = cudaGetLastError();

@@ -42,16 +42,16 @@
 //
 // What bounds it: instructions and the latency of the gathers.  Of 10^8
 // entries, K = 100, B = 64 (W beyond L2) a part-step's light rows without any
-// entry take 118 us, 92 M warp instructions at 0.66 per cycle and scheduler,
-// most of them Philox and the normals.  Against the gradient and the update
-// as two launches per side on two streams (before): 293 instead of 314 us a
-// part-step there; 43.9 instead of 45.8 us with 10^7 entries, K = 50, B = 32
-// (factors in L2); and one launch instead of four where launches count: a
-// sweep of 256 x 256 dense counts, K = 8, B = 4, and its read-back 29 instead
-// of 48 us.  Thresholds measured on the first two: mid rows up to 64 entries
-// 366 and 47 us (the columns of the first have 87 on average, and a block
-// each is too much), up to 512 291 and 63 us (a warp alone with such a row
-// is the part-step's tail).
+// entry take 114 us, 92 M warp instructions at 0.66 per cycle and scheduler,
+// most of them Philox and the normals (their rows come into L2 a warp's share
+// at a time: 118 us without).  Against the gradient and the update as two
+// launches per side on two streams (before): 281 instead of 314 us a part-step
+// there; 41.9 instead of 45.8 us with 10^7 entries, K = 50, B = 32 (factors in
+// L2); and one launch instead of four where launches count: a sweep of 256 x
+// 256 dense counts, K = 8, B = 4, and its read-back 31 instead of 48 us.
+// Thresholds measured on the first two, ms a sweep with light up to 16, mid up
+// to 128 and chunks of 512 18.0 and 1.34: 8, 128, 512: 18.3 and 1.43; 32, 128,
+// 512: 18.4 and 1.44; 16, 96, 384: 18.9 and 1.37; 16, 192, 768: 18.2 and 1.38.
 #include <algorithm>
 #include <cstring>
 #include <vector>
@@ -73,11 +73,12 @@ struct RowSide {
     const int32_t *ptr;        // this part's row offsets (absolute entry indices)
     const int32_t *idx;        // other index of each entry
     const float *val;
-    const int32_t *mid;        // this part's mid rows
-    const int2 *heavy;         // ... and chunks (row, number) of its heavy rows
+    const int4 *mid;           // this part's mid rows (row, first entry, entries, 0)
+    const int4 *heavy;         // ... and its heavy rows' chunks (row, first entry, entries, number)
     float *partial;            // a row of ldk sums per chunk
     int *arrived;              // per chunk: of a row's first one, the chunks done
     int n_rows, n_mid, n_heavy;   // zero when the factor is frozen
+    int far;                   // 1: the own factor is beyond L2
     float prior_a, prior_b;       // d log p(x)/dx = prior_a + prior_b * x
 };
 
@@ -120,6 +121,12 @@ __device__ __forceinline__ float4 shfl_xor4(const float4 a, int o)
 {
     return make_float4(__shfl_xor_sync(0xffffffffu, a.x, o), __shfl_xor_sync(0xffffffffu, a.y, o),
                        __shfl_xor_sync(0xffffffffu, a.z, o), __shfl_xor_sync(0xffffffffu, a.w, o));
+}
+
+// Bulk prefetch of `bytes` (a multiple of 16, 16-byte aligned) into L2.
+__device__ __forceinline__ void prefetch_l2(const void *src, uint32_t bytes)
+{
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" :: "l"(src), "r"(bytes) : "memory");
 }
 
 // A row read once, past L1 (which keeps the gathered rows).
@@ -367,11 +374,11 @@ __global__ void __launch_bounds__(kThreads, MINB) rows_kernel(const __grid_const
         const int sid = b < P.side[0].n_heavy ? 0 : 1;
         const RowSide &S = P.side[sid];
         if (sid) b -= P.side[0].n_heavy;
-        const int2 rec = __ldg(S.heavy + b);
-        const uint32_t row = (uint32_t)rec.x;
-        const uint32_t p0 = __ldg(S.ptr + row), p1 = __ldg(S.ptr + row + 1);
-        const int chunks = (int)((p1 - p0 + kChunk - 1) / kChunk);
-        const uint32_t c0 = p0 + (uint32_t)rec.y * kChunk, n = p1 - c0 < kChunk ? p1 - c0 : kChunk;
+        const int4 rec = __ldg(S.heavy + b);
+        const uint32_t row = (uint32_t)rec.x, all = (uint32_t)rec.z;
+        const int chunks = (int)((all + kChunk - 1) / kChunk);
+        const uint32_t at0 = (uint32_t)rec.w * kChunk, c0 = (uint32_t)rec.y + at0;
+        const uint32_t n = all - at0 < kChunk ? all - at0 : kChunk;
         r.load(S.X + (int64_t)row * P.ldk + 4 * l, in_last);
         constexpr uint32_t step = R * kWarps;       // entry i of team k of the block: i step + k
         const uint32_t k = warp * R + team;
@@ -406,7 +413,7 @@ __global__ void __launch_bounds__(kThreads, MINB) rows_kernel(const __grid_const
             if (q < P.ng) __stcg(reinterpret_cast<float4 *>(S.partial + (int64_t)b * P.ldk) + q, s);
             __threadfence();
             __syncthreads();
-            const int first = b - rec.y;
+            const int first = b - rec.w;
             if (threadIdx.x == 0) {
                 last = atomicAdd(S.arrived + first, 1) == chunks - 1;
                 if (last) S.arrived[first] = 0;
@@ -433,8 +440,8 @@ __global__ void __launch_bounds__(kThreads, MINB) rows_kernel(const __grid_const
         const RowSide &S = P.side[sid];
         const int at = (sid ? m - P.mid_blocks[0] : m) * kWarps + warp;
         if (at >= S.n_mid) return;
-        const uint32_t row = __ldg(S.mid + at);
-        const uint32_t p0 = __ldg(S.ptr + row), n = __ldg(S.ptr + row + 1) - p0;
+        const int4 rec = __ldg(S.mid + at);
+        const uint32_t row = (uint32_t)rec.x, p0 = (uint32_t)rec.y, n = (uint32_t)rec.z;
         const int64_t off = (int64_t)row * P.ldk + 4 * l;
         r.load(S.X + off, in_last);
         auto fetch = [&](uint32_t c, int &j, float &v) {   // entry i of team k: i R + k
@@ -494,6 +501,10 @@ __global__ void __launch_bounds__(kThreads, MINB) rows_kernel(const __grid_const
             vv = __ldg(S.val + e);
         }
     };
+    if (S.far && lane == 0 && row < n_rows) {
+        const uint32_t left = n_rows - row, mine = (uint32_t)(R * P.iters);
+        prefetch_l2(S.X + (int64_t)row * P.ldk, (left < mine ? left : mine) * (uint32_t)P.ldk * 4u);
+    }
     next_row();
     if (n <= light) fetch(p, n, 0, j, v);
     for (int it = 0; it < P.iters; ++it) {
@@ -534,12 +545,13 @@ struct RowKernel {
     RowFn fn;
 };
 
-// Lanes per team and groups per lane for ng float4 groups, entries together,
-// and blocks per SM to hold the registers to.  Up to 64 groups a lane has at
-// most two: with more groups in fewer lanes (8 x 4 for K = 100) the 114
-// registers leave 16 warps per SM, and the arithmetic of the update waits for
-// itself (part-step of 10^8 entries, K = 100: 387 us against 286 with 16 x 2
-// in 64 registers; 8 x 4 in 80 registers 328; 32 x 1 311).
+// Lanes per team and groups per lane for ng float4 groups, entries together
+// (light rows, others), and blocks per SM to hold the registers to.  Warps in
+// flight count most: 64 registers give 32 per SM, which two groups a lane and
+// two entries together fit.  Sweeps of 10^8 entries, K = 100 (and of 3 10^7,
+// BF16): 16 x 2 with 2 entries 18.0 (13.6) ms, with 4 in 80 registers 18.6
+// (14.3), 32 x 1 19.2 (14.2), 8 x 4 in 114 registers (16 warps) 24.7; of 10^7,
+// K = 50: 8 x 2 with 2 entries 1.34 ms, 16 x 1 with 4 1.37, with 2 1.46.
 template <bool BF>
 RowKernel pick_rows(int ng)
 {
@@ -547,7 +559,7 @@ RowKernel pick_rows(int ng)
     if (ng <= 2) return {2, rows_kernel<2, 1, 2, 2, BF, 4>};
     if (ng <= 4) return {4, rows_kernel<4, 1, 2, 4, BF, 4>};
     if (ng <= 8) return {8, rows_kernel<8, 1, 2, 4, BF, 4>};
-    if (ng <= 16) return {16, rows_kernel<16, 1, 4, 4, BF, 4>};
+    if (ng <= 16) return {8, rows_kernel<8, 2, 2, 2, BF, 4>};
     if (ng <= 32) return {16, rows_kernel<16, 2, 2, 2, BF, 4>};
     if (ng <= 48) return {16, rows_kernel<16, 3, 1, 2, BF, 3>};
     if (ng <= 64) return {32, rows_kernel<32, 2, 2, 2, BF, 4>};
@@ -616,6 +628,7 @@ psgld_status launch_rows(psgld_ctx *c, int part, int64_t t, const int64_t *t_dev
             S.Y16 = s == 0 ? c->H16[c->hcur] : c->W16[c->wcur];
             S.Xn16 = s == 0 ? c->W16[c->wcur ^ 1] : c->H16[c->hcur ^ 1];
         }
+        S.far = 4.0 * (double)n_rows * c->ldk > 64.0 * (1 << 20);
         S.ptr = L.ptr + (int64_t)part * n_rows;
         S.idx = L.idx;
         S.val = L.val;
