@@ -1094,6 +1094,10 @@ int64_t psgld_estimate_device_bytes(int64_t I, int64_t J, int32_t K, int32_t B, 
             bytes += (B * n_rows + 1) * 4 + nnz * (side == 0 ? 12 : 8) +
                      16 * (std::min(nnz / (light_row_for(I + J) + 1), B * n_rows) + max_chunks(nnz)) + (4 * ldk + 4) * std::min(max_chunks(nnz), max_chunks(cdiv(nnz, B)) + n_rows);
         }
+        // by units of entries: the B side's rows too, and the units' sums
+        const int ng = (K + 3) / 4;
+        if (step_by_units(I, J, ng, nnz, B))
+            bytes += nnz * 4 + 4 * (cdiv(cdiv(nnz, B), unit_entries(ng)) + 1) * ldk * 4;
         return bytes;
     }
     bytes += I * J * 4;   // the FP32 copy of V
@@ -1144,6 +1148,12 @@ void psgld_destroy(psgld_ctx *c)
     dev_free(c, c->sW.s); dev_free(c, c->sW.s2); dev_free(c, c->sH.s); dev_free(c, c->sH.s2);
     dev_free(c, c->red); dev_free(c, c->flag); dev_free(c, c->kflag); dev_free(c, c->t_dev);
     dev_free(c, c->eps_tab);
+    if (c->side_stream) {
+        cudaStreamSynchronize(c->side_stream);
+        cudaStreamDestroy(c->side_stream);
+    }
+    if (c->ev_fork) cudaEventDestroy(c->ev_fork);
+    if (c->ev_join) cudaEventDestroy(c->ev_join);
     if (c->capture_stream) cudaStreamDestroy(c->capture_stream);
     delete c;
     use_staging(-1);

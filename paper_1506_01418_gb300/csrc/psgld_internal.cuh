@@ -43,7 +43,10 @@ struct SideLayout {
     int32_t *ptr = nullptr;    // B*n_rows + 1 entry offsets (absolute)
     int32_t *idx = nullptr;    // other index of each entry
     float *val = nullptr;      // value of each entry
-    int32_t *own = nullptr;    // A side: own row of each entry (log-likelihood, RMSE)
+    int32_t *own = nullptr;    // own row of each entry (A side: also for log-likelihood and RMSE;
+                               // B side: contexts that step by units only)
+    std::vector<int64_t> part_first;   // B + 1: first entry of each part
+    float *unit_sums = nullptr;        // by units: head and tail sums, 2 x ldk per unit of a part
     // per part, the rows with more than light_row and at most kMidRow entries
     // in it (row, first entry, entries, 0), ascending, and the chunks of
     // kChunk entries of the rows with more (row, first entry, entries, number
@@ -150,6 +153,9 @@ struct psgld_ctx {
     cudaStream_t capture_stream = nullptr;
     int64_t *t_dev = nullptr;    // iteration counter read by graph replays
     int light_row = 0;           // most entries in a part of a row that one team takes (psgld_rows.cu)
+    bool units = false;          // sparse part-steps by units (psgld_units.cu)
+    cudaStream_t side_stream = nullptr;   // ... whose H^T side runs on a second stream
+    cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     int64_t t_dev_is = -1;       // its value after the work enqueued so far (-1: unknown)
     float2 *eps_tab = nullptr;   // captured sweeps with eps_t: (eps, sqrt(2 eps)) of each part-step
     psgld::BatchGraphs bgraphs;  // captured batch sweeps while this context leads a batch
@@ -240,6 +246,15 @@ psgld_status launch_part_step(psgld_ctx *c, int64_t t, const int64_t *t_dev,
 // The one launch of part `part` at iteration t (or *t_dev + t_add); does not
 // flip the context's buffers.
 psgld_status launch_rows(psgld_ctx *c, int part, int64_t t, const int64_t *t_dev, int64_t t_add, cudaStream_t st);
+// The same by units of consecutive entries (psgld_units.cu): whether a part
+// of nnz / B entries of I x J takes that form.
+bool step_by_units(int64_t I, int64_t J, int ngroups, int64_t nnz, int B);
+int unit_entries(int ngroups);
+int rows_groups(int ngroups);   // float4 groups, with padding, of a row in psgld_rows.cu
+psgld_status prepare_units(psgld_ctx *c);
+// `mid`, if given, is recorded between the gradients and the updates.
+psgld_status launch_units(psgld_ctx *c, int part, int64_t t, const int64_t *t_dev, int64_t t_add, cudaStream_t st,
+                          cudaEvent_t mid, unsigned rec_flags);
 // With gather_bf16 the part-step gathers BF16 copies of the factors (rows of
 // ldk rounded up to 8) and writes those of the new ones; built from the
 // current factors by build_gather_shadows (allocating them).

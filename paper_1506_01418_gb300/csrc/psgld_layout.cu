@@ -436,6 +436,7 @@ void free_layout(psgld_ctx *c)
     c->dense = false;
     c->ldv = 0;
     c->mtiles = 0;
+    c->units = false;
     c->has_data = false;
     c->N = 0;
     c->part_n.clear();
@@ -452,6 +453,11 @@ psgld_status build_layout(psgld_ctx *c, int64_t nnz, const int32_t *i_dev, const
     const int64_t I = c->I, J = c->J, n = nnz;
     const int B = c->B;
     c->light_row = light_row_for(I + J);
+    c->units = !c->opt.gather_bf16 && step_by_units(I, J, c->ngroups, n, B);
+    if (c->units) {
+        const psgld_status s = prepare_units(c);
+        if (s != PSGLD_OK) { dev_free(c, kept, st); return s; }
+    }
 
     const int64_t ntiles = std::max<int64_t>(1, (n + kSortTile - 1) / kSortTile);
     const int64_t nslots_max = (int64_t)B * std::max(I, J);
@@ -476,7 +482,7 @@ psgld_status build_layout(psgld_ctx *c, int64_t nnz, const int32_t *i_dev, const
         keep.add(&sd.ptr, nslots + 1);
         keep.add(&sd.idx, n);
         keep.add(&sd.val, n);
-        if (side == 0) keep.add(&sd.own, n);
+        if (side == 0 || c->units) keep.add(&sd.own, n);
         keep.add(&sd.mid, std::min(n / (c->light_row + 1), nslots));
         keep.add(&sd.heavy, max_chunks(n));
     }
@@ -574,6 +580,13 @@ psgld_status build_layout(psgld_ctx *c, int64_t nnz, const int32_t *i_dev, const
         if (side == 0) {
             c->part_n.resize(B);
             for (int p = 0; p < B; ++p) c->part_n[p] = at[p + 1] - at[p];
+        }
+        sd.part_first.assign(at, at + (B + 1));
+        if (c->units) {
+            int64_t units = 0;
+            for (int p = 0; p < B; ++p)
+                units = std::max(units, (at[p + 1] - at[p]) / unit_entries(c->ngroups) + 1);
+            chunk.add(&sd.unit_sums, 2 * units * c->ldk);
         }
         sd.mid_first.assign(at + (B + 1), at + 2 * (B + 1));
         sd.heavy_first.assign(at + 2 * (B + 1), at + 3 * (B + 1));

@@ -336,7 +336,7 @@ psgld_status launch_finish_sweep(psgld_ctx *c, bool acc, int64_t by, cudaStream_
     P.t = by > 0 ? c->t_dev : nullptr;
     P.by = by;
     const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>((P.n + 255) / 256, 152 * 16));
-    PSGLD_CK(c, launch_early(!c->opt.profile, finish_sweep_kernel, grid, P.n ? 256 : 32, 0, st, P));
+    PSGLD_CK(c, launch_early(!c->opt.profile && !c->units, finish_sweep_kernel, grid, P.n ? 256 : 32, 0, st, P));
     return PSGLD_OK;
 }
 

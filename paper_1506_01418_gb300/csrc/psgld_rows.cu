@@ -542,8 +542,12 @@ using RowFn = void (*)(RowParams);
 
 struct RowKernel {
     int T;
+    int groups;     // T lanes' float4 groups: ng and padding
     RowFn fn;
 };
+
+template <int T, int NG, int U, int UM, bool BF, int MINB>
+RowKernel rows() { return {T, T * NG, rows_kernel<T, NG, U, UM, BF, MINB>}; }
 
 // Lanes per team and groups per lane for ng float4 groups, entries together
 // (light rows, others), and blocks per SM to hold the registers to.  Warps in
@@ -552,19 +556,25 @@ struct RowKernel {
 // BF16): 16 x 2 with 2 entries 18.0 (13.6) ms, with 4 in 80 registers 18.6
 // (14.3), 32 x 1 19.2 (14.2), 8 x 4 in 114 registers (16 warps) 24.7; of 10^7,
 // K = 50: 8 x 2 with 2 entries 1.34 ms, 16 x 1 with 4 1.37, with 2 1.46.
+// A third group in 80 registers pays where it saves padding: 7 10^4 x 10^4,
+// 5 10^6 entries, B = 32 at K = 36: 4 x 3 886 us, 8 x 2 959; at K = 72, 96:
+// 8 x 3 1270, 1309, 16 x 2 1493, 1560; at K = 20, 32: 8 x 1 with 4 entries
+// 644, 654 us, with 2 704, 716.
 template <bool BF>
 RowKernel pick_rows(int ng)
 {
-    if (ng <= 1) return {1, rows_kernel<1, 1, 1, 1, BF, 4>};
-    if (ng <= 2) return {2, rows_kernel<2, 1, 2, 2, BF, 4>};
-    if (ng <= 4) return {4, rows_kernel<4, 1, 2, 4, BF, 4>};
-    if (ng <= 8) return {8, rows_kernel<8, 1, 2, 4, BF, 4>};
-    if (ng <= 16) return {8, rows_kernel<8, 2, 2, 2, BF, 4>};
-    if (ng <= 32) return {16, rows_kernel<16, 2, 2, 2, BF, 4>};
-    if (ng <= 48) return {16, rows_kernel<16, 3, 1, 2, BF, 3>};
-    if (ng <= 64) return {32, rows_kernel<32, 2, 2, 2, BF, 4>};
-    if (ng <= 96) return {32, rows_kernel<32, 3, 1, 2, BF, 3>};
-    return {32, rows_kernel<32, 4, 1, 2, BF, 2>};
+    if (ng <= 1) return rows<1, 1, 1, 1, BF, 4>();
+    if (ng <= 2) return rows<2, 1, 2, 2, BF, 4>();
+    if (ng <= 4) return rows<4, 1, 2, 4, BF, 4>();
+    if (ng <= 8) return rows<8, 1, 4, 4, BF, 4>();
+    if (ng <= 12) return rows<4, 3, 2, 2, BF, 3>();
+    if (ng <= 16) return rows<8, 2, 2, 2, BF, 4>();
+    if (ng <= 24) return rows<8, 3, 2, 2, BF, 3>();
+    if (ng <= 32) return rows<16, 2, 2, 2, BF, 4>();
+    if (ng <= 48) return rows<16, 3, 1, 2, BF, 3>();
+    if (ng <= 64) return rows<32, 2, 2, 2, BF, 4>();
+    if (ng <= 96) return rows<32, 3, 1, 2, BF, 3>();
+    return rows<32, 4, 1, 2, BF, 2>();
 }
 
 // BF16 copy of an n x ldk FP32 factor into rows of ld16 (padding zero)
@@ -586,6 +596,8 @@ __global__ void gather_copy_kernel(const float *__restrict__ X, int64_t n, int l
 int ld16_for(int ldk) { return 8 * ((ldk + 7) / 8); }
 
 }  // namespace
+
+int rows_groups(int ng) { return pick_rows<false>(ng).groups; }
 
 bool gather_bf16(const psgld_ctx *c) { return c->opt.gather_bf16 && !c->dense && c->W16[0] && c->H16[1]; }
 

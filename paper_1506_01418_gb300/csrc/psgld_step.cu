@@ -250,10 +250,16 @@ psgld_status launch_part_step(psgld_ctx *c, int64_t t, const int64_t *t_dev, int
         PSGLD_CK(c, cudaEventRecordWithFlags(c->ev_start[part], st, rec_flags));
     }
     if (!c->dense) {
-        const psgld_status rs = launch_rows(c, part, t, t_dev, t_add, st);
-        if (rs != PSGLD_OK) return rs;
-        // gradient and update are one launch, profiled as the gradient's
-        if (prof) PSGLD_CK(c, cudaEventRecordWithFlags(c->ev_mid[part], st, rec_flags));
+        // (the BF16 copies are written by the rows form alone)
+        if (c->units && !gather_bf16(c)) {
+            const psgld_status rs = launch_units(c, part, t, t_dev, t_add, st, prof ? c->ev_mid[part] : nullptr, rec_flags);
+            if (rs != PSGLD_OK) return rs;
+        } else {
+            const psgld_status rs = launch_rows(c, part, t, t_dev, t_add, st);
+            if (rs != PSGLD_OK) return rs;
+            // gradient and update are one launch, profiled as the gradient's
+            if (prof) PSGLD_CK(c, cudaEventRecordWithFlags(c->ev_mid[part], st, rec_flags));
+        }
     } else {
         UpdParams UP;
         fill_params(c, part, t, t_dev, t_add, UP);
