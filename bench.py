@@ -549,10 +549,10 @@ def run_ours(args, wl_name, wl):
                    "l2": "256 MB buffer written before every timed sweep",
                    "parallelism": f"replicas x{world}" if world > 1 else "single GPU"},
         "roofline": roofline,
-        # per sweep: B x (gradient + update) + 2 accumulate + advance t + set t
         # per part-step: the chain kernel and the update (tensor-core path),
-        # or one launch of both (sparse path); per sweep one more (posterior
-        # sums and the t counter)
+        # or one launch of both (sparse path; four with few entries per row,
+        # counted here as one); per sweep one more (posterior sums and the t
+        # counter)
         "gpu_launches": args.steps * ((2 if tensor_path(wl) else 1) * wl["B"] + 1),
         "clocks": clocks,
         "rmse_after": rmse,

@@ -18,9 +18,9 @@
 // item: the row's gradient (nothing for an empty row), noise, prior, step,
 // mirror; reads X_cur, writes X_next.
 //
-// Sweeps of 3 10^5 x 5000, 10^6 entries, B = 16, at K = 24, 32, 50, 100:
-// 450, 539, 855, 1559 us, with CUDA's logf, sqrtf and sincospif in the normals
-// 513, 625, 984, 1787; one launch of psgld_rows.cu: 700, 760, 1130, 1881.
+// Sweeps of 3 10^5 x 5000, 10^6 entries, B = 16, at K = 16, 50, 100: 355, 855,
+// 1559 us, with CUDA's logf, sqrtf and sincospif in the normals 404, 984, 1787;
+// one launch of psgld_rows.cu: 470, 1200, 1881.
 #include <algorithm>
 #include <cstring>
 #include <vector>
@@ -519,7 +519,7 @@ int unit_entries(int ngroups) { return shape_for(ngroups).E; }
 //   warp's walk over a row with a hundred entries.  1600 rows, 25 000 entries,
 //   K = 128, 200: 49 / 66, 81 / 115; 35 000 rows, 31 000 entries, 429 / 455,
 //   584 / 763; 28 000 rows, 62 000 entries, 487 / 457, 715 / 784;
-//   K = 300: 25 000 entries 137 / 123, 2500 60 / 117.
+//   K = 300: 25 000 entries 137 / 123, 2500 59 / 117.
 // All indices in 32 bits.
 bool step_by_units(int64_t I, int64_t J, int ngroups, int64_t nnz, int B)
 {
