@@ -37,9 +37,13 @@ constexpr size_t kHalf = 4 << 20;      // staging: two halves, one filled while 
 constexpr size_t kSlice = 256 << 10;   // bytes a thread copies at a time
 constexpr size_t kDirect = 1 << 20;    // read-backs up to this go without staging
 // and up to this the sums come over and are divided on the host, which saves
-// four launches: 389 x 8 moments 117 us formed on the device; at 3896 x 8
-// (500 KB) both take 130
-constexpr size_t kHost = 256 << 10;
+// four launches.  Moments of 0.4, 0.6, 0.9 MB: 101, 121, 148 us on the host,
+// 125, 129, 135 formed on the device; of 1.3 and 1.8 MB through staging 192 and
+// 229, divided on the host 186 and 235.
+constexpr size_t kHost = 768 << 10;
+// bytes per helping thread: of 1.8 MB with seven 666 us, with none 229; of 8 MB
+// 866, 776 with one, 897 with none; of 40 MB 1509, 3562 with none
+constexpr int64_t kPerHelper = 4 << 20;
 constexpr unsigned kThreads = 8;
 
 // One staging area for the process, used by one read-back at a time, given
@@ -214,7 +218,7 @@ psgld_status read_moments(psgld_ctx *c, double *const (&out)[2][2])
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
     {
         const unsigned hw = std::max(1u, std::thread::hardware_concurrency());
-        Crew crew(std::min(kThreads, hw) - 1);
+        Crew crew((unsigned)std::min<int64_t>(std::min(kThreads, hw) - 1, total / kPerHelper));
         auto fetch = [&](size_t k) {
             e = form(c, pieces[k], st);
             if (e == cudaSuccess)
