@@ -27,6 +27,7 @@
 #include <utility>
 
 #include "psgld_internal.cuh"
+#include "psgld_slots.cuh"
 
 namespace psgld {
 
@@ -591,10 +592,10 @@ psgld_status build_layout(psgld_ctx *c, int64_t nnz, const int32_t *i_dev, const
         }
         sd.part_first.assign(at, at + (B + 1));
         if (c->units) {
-            int64_t units = 0;
+            int64_t floats = 0;
             for (int p = 0; p < B; ++p)
-                units = std::max(units, (at[p + 1] - at[p]) / unit_entries(c->ngroups) + 1);
-            chunk.add(&sd.unit_sums, 2 * units * c->ldk);
+                floats = std::max(floats, slot_floats(at[p + 1] - at[p], unit_entries(c->ngroups), c->ldk));
+            chunk.add(&sd.unit_sums, floats);
         }
         sd.mid_first.assign(at + (B + 1), at + 2 * (B + 1));
         sd.heavy_first.assign(at + 2 * (B + 1), at + 3 * (B + 1));

@@ -25,6 +25,7 @@
 #include <cstring>
 #include <vector>
 
+#include "psgld_slots.cuh"
 #include "psgld_update.cuh"
 
 namespace psgld {
@@ -307,8 +308,8 @@ __device__ __forceinline__ bool grad_unit(const GradParams &P, int64_t u, const 
                 acc[g].w += __shfl_xor_sync(0xffffffffu, acc[g].w, o);
             }
         const int row = ow[0];
-        float *dst = prev_own == row ? Sd.partial + (2 * u) * (int64_t)ldk
-                   : next_own == row ? Sd.partial + (2 * u + 1) * (int64_t)ldk
+        float *dst = prev_own == row ? Sd.partial + head_slot(u, ldk)
+                   : next_own == row ? Sd.partial + tail_slot(u, ldk)
                                      : Sd.Gout + (int64_t)row * ldk;
         if (sub == 0) {
 #pragma unroll
@@ -333,8 +334,8 @@ __device__ __forceinline__ bool grad_unit(const GradParams &P, int64_t u, const 
                     if (q < ng) axpy4(acc[g], es_, ys4(ys, sl, q, lds));
                 }
             }
-            float *dst = (k == 0 && prev_own == row) ? Sd.partial + (2 * u) * (int64_t)ldk
-                       : (k == nseg - 1 && next_own == row) ? Sd.partial + (2 * u + 1) * (int64_t)ldk
+            float *dst = (k == 0 && prev_own == row) ? Sd.partial + head_slot(u, ldk)
+                       : (k == nseg - 1 && next_own == row) ? Sd.partial + tail_slot(u, ldk)
                                                              : Sd.Gout + (int64_t)row * ldk;
 #pragma unroll
             for (int g = 0; g < NG; ++g) {
@@ -382,8 +383,8 @@ __global__ void __launch_bounds__(kGradThreads) grad_kernel(const __grid_constan
     }
 }
 
-// One (row, float4 group) item of factor SID (0 = W, 1 = H^T), in 32-bit
-// index arithmetic (step_by_units checks the sizes).
+// One (row, float4 group) item of factor SID (0 = W, 1 = H^T): items and
+// factor offsets in 32 bits (step_by_units checks the sizes), slots in 64.
 template <int SID>
 __device__ __forceinline__ void update_item32(const UpdParams &P, uint32_t item, float eps, float sd,
                                               uint32_t t_lo, uint32_t t_hi)
@@ -402,19 +403,18 @@ __device__ __forceinline__ void update_item32(const UpdParams &P, uint32_t item,
             g = ldg4(Sd.Gin + off);
         } else {
             // the row's first unit's tail slot, then the later units' head slots, in unit order
-            const uint32_t ldk = (uint32_t)P.ldk;
-            g = __ldcg(reinterpret_cast<const float4 *>(Sd.partial + (2u * u0 + 1u) * ldk + 4u * q));
+            g = __ldcg(reinterpret_cast<const float4 *>(Sd.partial + tail_slot(u0, P.ldk) + 4u * q));
             const float *hp = Sd.partial + 4u * q;
             int uu = u0 + 1;
             for (; uu + 8 <= u1 + 1; uu += 8) {   // eight independent loads in flight
                 float4 v[8];
 #pragma unroll
                 for (int w = 0; w < 8; ++w)
-                    v[w] = __ldcg(reinterpret_cast<const float4 *>(hp + 2u * (uint32_t)(uu + w) * ldk));
+                    v[w] = __ldcg(reinterpret_cast<const float4 *>(hp + head_slot(uu + w, P.ldk)));
 #pragma unroll
                 for (int w = 0; w < 8; ++w) add4(g, v[w]);
             }
-            for (; uu <= u1; ++uu) add4(g, __ldcg(reinterpret_cast<const float4 *>(hp + 2u * (uint32_t)uu * ldk)));
+            for (; uu <= u1; ++uu) add4(g, __ldcg(reinterpret_cast<const float4 *>(hp + head_slot(uu, P.ldk))));
         }
     }
     const float4 z = dev::normals4(dev::philox(make_uint4(q, row, t_lo, (t_hi << 1) | (uint32_t)SID), P.noise.rk0,
@@ -520,11 +520,11 @@ int unit_entries(int ngroups) { return shape_for(ngroups).E; }
 //   K = 128, 200: 49 / 66, 81 / 115; 35 000 rows, 31 000 entries, 429 / 455,
 //   584 / 763; 28 000 rows, 62 000 entries, 487 / 457, 715 / 784;
 //   K = 300: 25 000 entries 137 / 123, 2500 59 / 117.
-// All indices in 32 bits.
+// Items and factor offsets in 32 bits.
 bool step_by_units(int64_t I, int64_t J, int ngroups, int64_t nnz, int B)
 {
     const int64_t rows = I + J, items = rows * ngroups, lim = (1ll << 31) - 1;
-    if (items > lim || std::max(I, J) * 4 * ngroups > lim || 2 * (nnz / B + 1) * 4 * ngroups > lim) return false;
+    if (items > lim || std::max(I, J) * 4 * ngroups > lim) return false;
     if (ngroups > 24 && nnz < (ngroups <= 64 ? 1536ll : 128ll) * ngroups * B) return true;
     if (ngroups <= 2 || items <= (1 << 19)) return false;
     const double padding = (double)rows_groups(ngroups) / ngroups - 1.0;
