@@ -974,13 +974,10 @@ psgld_status psgld_batch_sweep(psgld_ctx *const *ctxs, int32_t n, int32_t n_swee
         for (int b = 0; b < B && r == PSGLD_OK; ++b) {
             const size_t row = (size_t)(q * B + b) * n;
             if (prof) r = record(c0->ev_start[b]);
-            bool late = false;
-            for (int g = 0; g < ng && r == PSGLD_OK; ++g) {
+            for (int g = 0; g < ng && r == PSGLD_OK; ++g)
                 r = launch_dense_batch(c0, keys[g], d + off_dp + dp * (row + gbeg[g]),
                                        reinterpret_cast<const int *>(d + off_cta) + 2 * (gbeg[g] + g),
-                                       gbeg[g + 1] - gbeg[g], g_ctas[g], late, ss);
-                late = late || g_ctas[g] > 0;
-            }
+                                       gbeg[g + 1] - gbeg[g], g_ctas[g], ss);
             if (r == PSGLD_OK && prof) r = record(c0->ev_mid[b]);
             if (r == PSGLD_OK)
                 r = launch_update_batch(c0, d + off_up + upb * row,

@@ -860,7 +860,7 @@ __device__ __forceinline__ const Params &ctx_of(const Params &P0, const Src &src
 // The kernel body.  P0 gives what is uniform over the launch (K width,
 // ring depths); each item reads its own context's parameters.
 template <typename VT, int PM, bool BATCH>
-__device__ __forceinline__ void chain_body(const Params &P0, const Src src, int total_items, const bool late)
+__device__ __forceinline__ void chain_body(const Params &P0, const Src src, int total_items)
 {
     extern __shared__ __align__(1024) unsigned char sm_raw[];
     // the swizzled operand tiles need 1024-byte alignment (1 KB of slack is allocated)
@@ -900,9 +900,7 @@ __device__ __forceinline__ void chain_body(const Params &P0, const Src src, int 
     __syncthreads();
     fence_after();
     const uint32_t tmem = S->tmem;
-    // a late launch's inputs are complete already (launch_dense_batch): it
-    // waits at its end, so that the launch after it waits for both
-    if (!late) dev::wait_prior();
+    dev::wait_prior();
     dev::let_next();
 
     if (warp == 0) {
@@ -1140,7 +1138,6 @@ __device__ __forceinline__ void chain_body(const Params &P0, const Src src, int 
         __syncwarp();
     }
 
-    if (late) dev::wait_prior();
     fence_before();
     __syncthreads();
     fence_after();
@@ -1160,17 +1157,16 @@ __device__ __forceinline__ void chain_body(const Params &P0, const Src src, int 
 template <typename VT, int PM>
 __global__ void __launch_bounds__(kThreads, 1) chain_kernel(const __grid_constant__ Params P)
 {
-    chain_body<VT, PM, false>(P, Src{nullptr, nullptr, nullptr, 1, 0}, P.items, false);
+    chain_body<VT, PM, false>(P, Src{nullptr, nullptr, nullptr, 1, 0}, P.items);
 }
 
 // Many contexts of one K width, V type and power in one persistent launch.
 template <typename VT, int PM>
 __global__ void __launch_bounds__(kThreads, 1)
-chain_batch_kernel(const unsigned char *tab, size_t stride, const int *rows_start, const int *cols_start, int n,
-                   int late)
+chain_batch_kernel(const unsigned char *tab, size_t stride, const int *rows_start, const int *cols_start, int n)
 {
     chain_body<VT, PM, true>(*reinterpret_cast<const Params *>(tab), Src{tab, rows_start, cols_start, n, stride},
-                             __ldg(rows_start + n) + __ldg(cols_start + n), late != 0);
+                             __ldg(rows_start + n) + __ldg(cols_start + n));
 }
 
 }  // namespace two_sided_rc
@@ -2693,7 +2689,7 @@ int fill_dense_param(const psgld_ctx *c, int part, void *dst, int *first_items)
 }
 
 psgld_status launch_dense_batch(psgld_ctx *c0, int key, const void *params, const int *cta_start, int n,
-                                int total, bool late, cudaStream_t st)
+                                int total, cudaStream_t st)
 {
     const bool early = !c0->opt.profile;
     const unsigned char *tab = static_cast<const unsigned char *>(params);
@@ -2716,7 +2712,7 @@ psgld_status launch_dense_batch(psgld_ctx *c0, int key, const void *params, cons
         if (c0->opt.batch_ctas > 0) grid = std::min(grid, (int)c0->opt.batch_ctas);
         if (grid > 0)
             PSGLD_CK(c0, launch_early(early, fn, (unsigned)grid, two_sided_rc::kThreads, smem, st, tab, stride, cta_start,
-                                      cta_start + n + 1, n, early && late ? 1 : 0));
+                                      cta_start + n + 1, n));
         return PSGLD_OK;
     }
     if (key >= 8192) {

@@ -307,11 +307,8 @@ int dense_batch_key(const psgld_ctx *c);
 int dense_batch_length(const psgld_ctx *c);
 size_t dense_param_bytes();
 int fill_dense_param(const psgld_ctx *c, int part, void *dst, int *first_items);
-// late (not the part's first gradient launch): the launch waits for the one
-// before it at its end instead of its start -- the two share nothing, and
-// that one has waited for the update before them.
 psgld_status launch_dense_batch(psgld_ctx *c0, int key, const void *params, const int *cta_start, int n,
-                                int total, bool late, cudaStream_t st);
+                                int total, cudaStream_t st);
 // Update of part `part` at iteration *t_dev + t_add (t_dev: the context's
 // device counter); does not flip the context's buffers.
 size_t upd_param_bytes();

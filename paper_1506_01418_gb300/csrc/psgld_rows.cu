@@ -363,8 +363,8 @@ __global__ void __launch_bounds__(kThreads, MINB) rows_kernel(const __grid_const
     const int l = lane & (T - 1), team = lane / T;
     const bool in_last = l + (NG - 1) * T < P.ng;
     const int n_heavy = P.side[0].n_heavy + P.side[1].n_heavy;
-    dev::let_next();
     dev::wait_prior();
+    dev::let_next();
     if (P.wait_polls && !gather_wait_check(P, P.side[P.side[0].n_rows ? 0 : 1])) return;
     const Clock clk = read_clock(P.noise);
     Row<T, NG> r;
