@@ -223,7 +223,7 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi)
 // 128 x KP K-major BF16 tile, zero padded; half h of the K range.  Returns
 // the largest |x| this thread staged.
 template <int KP>
-__device__ __forceinline__ float stage_rows(unsigned char *tile, const float *__restrict__ X, int64_t src_row,
+__device__ __forceinline__ float stage_rows(unsigned char *tile, const float *X, int64_t src_row,
                                             int64_t end, int K, int ldk, int r, int h)
 {
     const bool v = src_row < end;
@@ -232,7 +232,7 @@ __device__ __forceinline__ float stage_rows(unsigned char *tile, const float *__
 #pragma unroll
     for (int k = h * kHalf; k < (h + 1) * kHalf; k += 4) {
         float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (v && k < K) x = __ldg(reinterpret_cast<const float4 *>(X + src_row * ldk + k));
+        if (v && k < K) x = *reinterpret_cast<const float4 *>(X + src_row * ldk + k);
         const float a = x.x, b = k + 1 < K ? x.y : 0.f, c = k + 2 < K ? x.z : 0.f,
                     d = k + 3 < K ? x.w : 0.f;
         amax = fmaxf(amax, fmaxf(fmaxf(fabsf(a), fabsf(b)), fmaxf(fabsf(c), fabsf(d))));
@@ -260,7 +260,7 @@ __device__ __forceinline__ uint32_t cm8_off(int r, int k, int KD)
 // The same row as stage_rows, times inv_s, into a 128 x KD E4M3 tile (KD =
 // KP rounded up to 32, one MMA K step), zero padded; half h of the K range.
 template <int KD>
-__device__ __forceinline__ void stage_rows_e4m3(unsigned char *tile, const float *__restrict__ X,
+__device__ __forceinline__ void stage_rows_e4m3(unsigned char *tile, const float *X,
                                                 int64_t src_row, int64_t end, int K, int ldk, int r, int h,
                                                 float inv_s)
 {
@@ -273,7 +273,7 @@ __device__ __forceinline__ void stage_rows_e4m3(unsigned char *tile, const float
         for (int q = 0; q < 4; ++q) {
             const int kk = k + 4 * q;
             float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (v && kk < K) x = __ldg(reinterpret_cast<const float4 *>(X + src_row * ldk + kk));
+            if (v && kk < K) x = *reinterpret_cast<const float4 *>(X + src_row * ldk + kk);
             w[q] = pack_e4m3x4(x.x * inv_s, kk + 1 < K ? x.y * inv_s : 0.f, kk + 2 < K ? x.z * inv_s : 0.f,
                                kk + 3 < K ? x.w * inv_s : 0.f);
         }
@@ -1404,7 +1404,7 @@ __device__ __forceinline__ bool wait32(Bars *S, uint64_t *b, uint32_t parity)
     return ok;
 }
 
-// 16 bytes of data read once (no L1 allocation)
+// 16 bytes of V, read once (no L1 allocation)
 __device__ __forceinline__ uint4 ldg_stream(const void *p)
 {
     uint4 r;
@@ -2256,7 +2256,7 @@ ChainRcFn pick_chain_rc(bool vb, int pm)
     return f[vb ? 1 : 0][pm];
 }
 
-using ChainRcBatchFn = void (*)(const unsigned char *, size_t, const int *, const int *, int, int);
+using ChainRcBatchFn = void (*)(const unsigned char *, size_t, const int *, const int *, int);
 
 ChainRcBatchFn pick_chain_batch_rc(bool vb, int pm)
 {

@@ -195,8 +195,13 @@ cudaError_t wait_enqueued(psgld_ctx *c);
 // dev::wait_prior, so that the launch itself, and what a kernel does before
 // it reads anything, cost nothing between two kernels of a sweep.  Every
 // kernel launched this way calls dev::wait_prior before it touches memory
-// that an earlier kernel writes, or that one reads and it writes.  With
-// `early` false (profiling: events between the kernels) a plain launch.
+// that an earlier kernel writes, or that one reads and it writes, and calls
+// dev::let_next only after that.  What an earlier kernel of a sweep writes
+// (factors, their copies, gradients, the step-size table) it reads by
+// ordinary loads: its lifetime overlaps the writes, and the read-only path
+// (__ldg, ld.global.nc) is for memory that nothing writes meanwhile, here
+// the data, the layout and the batch tables.  With `early` false (profiling:
+// events between the kernels) a plain launch.
 template <class... KA, class... A>
 cudaError_t launch_early(bool early, void (*kernel)(KA...), unsigned grid, int threads, size_t smem,
                          cudaStream_t st, A &&...args)

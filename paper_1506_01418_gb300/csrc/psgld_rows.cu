@@ -133,8 +133,17 @@ __device__ __forceinline__ void prefetch_l2(const void *src, uint32_t bytes)
 __device__ __forceinline__ float4 ld_stream(const float *p)
 {
     float4 v;
-    asm volatile("ld.global.nc.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];"
-                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+    asm volatile("ld.global.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p) : "memory");
+    return v;
+}
+
+// From L2: sums that other blocks of this launch wrote.
+__device__ __forceinline__ float4 ld_l2(const float *p)
+{
+    float4 v;
+    asm volatile("ld.global.cg.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p) : "memory");
     return v;
 }
 
@@ -205,11 +214,11 @@ struct Source {
         for (int g = 0; g < NG; ++g) {
             const char *at = g + 1 < NG || NG == 1 ? row + g * T * kGroup : last + (uint64_t)j * pitch;
             if constexpr (BF) {
-                const uint2 w = __ldg(reinterpret_cast<const uint2 *>(at));
+                const uint2 w = *reinterpret_cast<const uint2 *>(at);
                 y[g] = make_float4(__uint_as_float(w.x << 16), __uint_as_float(w.x & 0xFFFF0000u),
                                    __uint_as_float(w.y << 16), __uint_as_float(w.y & 0xFFFF0000u));
             } else {
-                y[g] = __ldg(reinterpret_cast<const float4 *>(at));
+                y[g] = *reinterpret_cast<const float4 *>(at);
             }
         }
     }
@@ -283,7 +292,7 @@ __device__ __forceinline__ Clock read_clock(const StepNoise &N)
     c.eps = N.eps;
     c.sd = N.sd;
     if (N.eps_tab) {
-        const float2 e = __ldg(N.eps_tab + (N.t_add - 1));
+        const float2 e = N.eps_tab[N.t_add - 1];
         c.eps = e.x;
         c.sd = e.y;
     }
@@ -424,12 +433,12 @@ __global__ void __launch_bounds__(kThreads, MINB) rows_kernel(const __grid_const
             if (q < P.ng) {
                 s = dev::zero4();
                 for (int i = 0; i < chunks; ++i)
-                    dev::add4(s, __ldcg(reinterpret_cast<const float4 *>(S.partial + (int64_t)(first + i) * P.ldk) + q));
+                    dev::add4(s, ld_l2(S.partial + (int64_t)(first + i) * P.ldk + 4 * q));
             }
         }
         if (q < P.ng) {
             const int64_t off = (int64_t)row * P.ldk + 4 * q;
-            store_group<BF>(P, S, sid, clk, row, q, dev::ldg4(S.X + off), s, S.Xn + off);
+            store_group<BF>(P, S, sid, clk, row, q, dev::ld4(S.X + off), s, S.Xn + off);
         }
         return;
     }

@@ -53,7 +53,7 @@ __device__ __forceinline__ int64_t read_step(const UpdParams &P, float &eps, flo
     eps = N.eps;
     sd = N.sd;
     if (N.eps_tab) {
-        const float2 e = __ldg(N.eps_tab + (N.t_add - 1));
+        const float2 e = N.eps_tab[N.t_add - 1];
         eps = e.x;
         sd = e.y;
     } else if (P.eps_poly) {
@@ -75,10 +75,10 @@ __device__ __forceinline__ void update_item(const UpdParams &P, int64_t item, fl
     const int64_t row = P.div_magic ? (int64_t)__umulhi((uint32_t)item, P.div_magic) : item / ng;
     const int q = (int)(item - row * ng);
     const int64_t off = row * ldk + 4 * q;
-    const float4 x = dev::ldg4(Sd.X_cur + off);
+    const float4 x = dev::ld4(Sd.X_cur + off);
     // G, or the sum in M-tile order of the block's partial arrays
-    float4 g = dev::ldg4(Sd.Gin + off);
-    for (int h = 1; h < Sd.gparts; ++h) dev::add4(g, dev::ldg4(Sd.Gin + h * Sd.gstride + off));
+    float4 g = dev::ld4(Sd.Gin + off);
+    for (int h = 1; h < Sd.gparts; ++h) dev::add4(g, dev::ld4(Sd.Gin + h * Sd.gstride + off));
     const float4 z = dev::box_muller4(dev::philox(make_uint4((uint32_t)q, (uint32_t)row, t_lo, (t_hi << 1) | (uint32_t)SID),
                                                   P.noise.rk0, P.noise.rk1));
     float4 o = dev::langevin4(P.noise, Sd.prior_a, Sd.prior_b, x, g, z, eps, sd);
@@ -130,10 +130,10 @@ __device__ __forceinline__ void update_item_dense32(const UpdParams &P, uint32_t
     const uint32_t row = P.div_magic ? __umulhi(item, P.div_magic) : item / ng;
     const uint32_t q = item - row * ng;
     const uint32_t off = row * (uint32_t)P.ldk + 4u * q;
-    const float4 x = dev::ldg4(Sd.X_cur + off);
+    const float4 x = dev::ld4(Sd.X_cur + off);
     // G, or the sum in M-tile order of the block's partial arrays
-    float4 g = dev::ldg4(Sd.Gin + off);
-    for (int h = 1; h < Sd.gparts; ++h) dev::add4(g, dev::ldg4(Sd.Gin + (uint32_t)h * (uint32_t)Sd.gstride + off));
+    float4 g = dev::ld4(Sd.Gin + off);
+    for (int h = 1; h < Sd.gparts; ++h) dev::add4(g, dev::ld4(Sd.Gin + (uint32_t)h * (uint32_t)Sd.gstride + off));
     const float4 z = dev::box_muller4(dev::philox(make_uint4(q, row, t_lo, (t_hi << 1) | (uint32_t)SID),
                                                   P.noise.rk0, P.noise.rk1));
     float4 o = dev::langevin4(P.noise, Sd.prior_a, Sd.prior_b, x, g, z, eps, sd);

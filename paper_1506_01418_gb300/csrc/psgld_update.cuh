@@ -28,6 +28,10 @@ void fill_noise(const psgld_ctx *c, int part, int64_t t, const int64_t *t_dev, i
 
 namespace dev {
 
+// An ordinary load: for factors and gradients in kernels that launch_early
+// starts (see there).  ldg4 is for plain launches.
+__device__ __forceinline__ float4 ld4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
+
 __device__ __forceinline__ float4 ldg4(const float *p) { return __ldg(reinterpret_cast<const float4 *>(p)); }
 
 __device__ __forceinline__ float4 zero4() { return make_float4(0.f, 0.f, 0.f, 0.f); }
