@@ -2659,6 +2659,8 @@ int dense_batch_key(const psgld_ctx *c)
     return 0;
 }
 
+bool dense_batch_beside(int key) { return key >= 4096 && key < 8192; }
+
 size_t dense_param_bytes()
 {
     const size_t m = std::max({sizeof(DenseParams), sizeof(two_sided::Params), sizeof(two_sided_rc::Params)});
@@ -2689,9 +2691,8 @@ int fill_dense_param(const psgld_ctx *c, int part, void *dst, int *first_items)
 }
 
 psgld_status launch_dense_batch(psgld_ctx *c0, int key, const void *params, const int *cta_start, int n,
-                                int total, cudaStream_t st)
+                                int total, bool early, cudaStream_t st)
 {
-    const bool early = !c0->opt.profile;
     const unsigned char *tab = static_cast<const unsigned char *>(params);
     const size_t stride = dense_param_bytes();
     if (key >= 4096 && key < 8192) {

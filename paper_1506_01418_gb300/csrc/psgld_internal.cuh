@@ -154,7 +154,7 @@ struct psgld_ctx {
     int64_t *t_dev = nullptr;    // iteration counter read by graph replays
     int light_row = 0;           // most entries in a part of a row that one team takes (psgld_rows.cu)
     bool units = false;          // sparse part-steps by units (psgld_units.cu)
-    cudaStream_t side_stream = nullptr;   // ... whose H^T side runs on a second stream
+    cudaStream_t side_stream = nullptr;   // second stream (units: the H^T side; batches: kernel variants)
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     int64_t t_dev_is = -1;       // its value after the work enqueued so far (-1: unknown)
     float2 *eps_tab = nullptr;   // captured sweeps with eps_t: (eps, sqrt(2 eps)) of each part-step
@@ -187,6 +187,13 @@ void dev_free(psgld_ctx *c, void *p, cudaStream_t st = nullptr);
 // rest of the stream), or syncs the last stream if no event was recorded.
 void mark_enqueued(psgld_ctx *c, cudaStream_t st);
 cudaError_t wait_enqueued(psgld_ctx *c);
+
+// ---- a second stream ---------------------------------------------------------
+// The context's side stream and its events, made on first use; work forked
+// onto it from st, and st made to wait for it (graph edges inside a capture).
+psgld_status side_stream(psgld_ctx *c);
+psgld_status fork_side(psgld_ctx *c, cudaStream_t st);
+psgld_status join_side(psgld_ctx *c, cudaStream_t st);
 
 // ---- launches that start early ---------------------------------------------
 // Programmatic dependent launch: the kernel's blocks may become resident
@@ -312,14 +319,18 @@ int dense_batch_key(const psgld_ctx *c);
 int dense_batch_length(const psgld_ctx *c);
 size_t dense_param_bytes();
 int fill_dense_param(const psgld_ctx *c, int part, void *dst, int *first_items);
+// early: launch_early (else a plain launch).
 psgld_status launch_dense_batch(psgld_ctx *c0, int key, const void *params, const int *cta_start, int n,
-                                int total, cudaStream_t st);
+                                int total, bool early, cudaStream_t st);
+// Whether the launches of a key wait for nothing but their own copies: such
+// ones may run beside another of the same part, which shares nothing.
+bool dense_batch_beside(int key);
 // Update of part `part` at iteration *t_dev + t_add (t_dev: the context's
 // device counter); does not flip the context's buffers.
 size_t upd_param_bytes();
 int64_t fill_upd_param(psgld_ctx *c, int part, const int64_t *t_dev, int64_t t_add, void *dst);
 psgld_status launch_update_batch(psgld_ctx *c0, const void *params, const int64_t *item_start, int n,
-                                 int64_t total_items, cudaStream_t st);
+                                 int64_t total_items, bool early, cudaStream_t st);
 // Posterior sums: a context takes the sample when (*t_dev - t0) / B >= acc_from.
 size_t acc_param_bytes();
 int64_t fill_acc_param(psgld_ctx *c, int64_t t0, int64_t acc_from, void *dst);

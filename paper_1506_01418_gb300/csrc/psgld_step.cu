@@ -353,12 +353,12 @@ int64_t fill_upd_param(psgld_ctx *c, int part, const int64_t *t_dev, int64_t t_a
 }
 
 psgld_status launch_update_batch(psgld_ctx *c0, const void *params, const int64_t *item_start, int n,
-                                 int64_t total_items, cudaStream_t st)
+                                 int64_t total_items, bool early, cudaStream_t st)
 {
     const int64_t cap = c0->opt.batch_update_blocks > 0 ? c0->opt.batch_update_blocks : 152 * 16;
     const int grid = (int)std::min<int64_t>((total_items + kThreads - 1) / kThreads, cap);
     if (grid > 0)
-        PSGLD_CK(c0, launch_early(!c0->opt.profile, update_batch_kernel, (unsigned)grid, kThreads, 0, st,
+        PSGLD_CK(c0, launch_early(early, update_batch_kernel, (unsigned)grid, kThreads, 0, st,
                                   static_cast<const UpdParams *>(params), item_start, n));
     return PSGLD_OK;
 }

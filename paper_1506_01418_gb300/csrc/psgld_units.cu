@@ -567,12 +567,7 @@ psgld_status prepare_units(psgld_ctx *c)
     const GradFn fn = pick_grad(sh);
     if (!fn) return fail(c, PSGLD_ERR_ARG, "unsupported K");
     PSGLD_CK(c, cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)grad_smem(sh)));
-    if (!c->side_stream) {
-        PSGLD_CK(c, cudaStreamCreateWithFlags(&c->side_stream, cudaStreamNonBlocking));
-        PSGLD_CK(c, cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming));
-        PSGLD_CK(c, cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming));
-    }
-    return PSGLD_OK;
+    return side_stream(c);
 }
 
 psgld_status launch_units(psgld_ctx *c, int part, int64_t t, const int64_t *t_dev, int64_t t_add, cudaStream_t st,
@@ -665,16 +660,14 @@ psgld_status launch_units(psgld_ctx *c, int part, int64_t t, const int64_t *t_de
     }
     const bool l2_fit = 4.0 * (double)(c->I + c->J) * c->ldk <= 64.0 * (1 << 20);
     if (!l2_fit) gradient(0, st, true);
-    PSGLD_CK(c, cudaEventRecord(c->ev_fork, st));
-    PSGLD_CK(c, cudaStreamWaitEvent(c->side_stream, c->ev_fork, 0));
+    const psgld_status fs = fork_side(c, st);
+    if (fs != PSGLD_OK) return fs;
     gradient(1, c->side_stream, !l2_fit);
     update(1, c->side_stream);
     if (l2_fit) gradient(0, st, false);
     update(0, st);
     PSGLD_CK(c, cudaGetLastError());
-    PSGLD_CK(c, cudaEventRecord(c->ev_join, c->side_stream));
-    PSGLD_CK(c, cudaStreamWaitEvent(st, c->ev_join, 0));
-    return PSGLD_OK;
+    return join_side(c, st);
 }
 
 }  // namespace psgld
