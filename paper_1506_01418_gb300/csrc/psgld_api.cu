@@ -485,8 +485,10 @@ psgld_status psgld_set_data_coo(psgld_ctx *c, int64_t nnz, const int32_t *i, con
     if (nnz > 0 && (!i || !j || !v)) return fail(c, PSGLD_ERR_ARG, "null entry array");
     cudaStream_t st = (cudaStream_t)stream;
     destroy_graphs(c);
-    // entries already on this device are read where they are
+    // entries already on this device are read where they are, if a kernel can
+    // (a copy takes any address, a 4-byte load an aligned one)
     auto here = [&](const void *p) {
+        if (reinterpret_cast<uintptr_t>(p) % 4 != 0) return false;
         cudaPointerAttributes at{};
         const bool dev = p && cudaPointerGetAttributes(&at, p) == cudaSuccess && at.type == cudaMemoryTypeDevice &&
                          at.device == c->device;
