@@ -762,6 +762,9 @@ psgld_status psgld_set_state(psgld_ctx *c, const double *sW, const double *sW2, 
     // the padding columns (K .. ldk-1) stay as they are: zero
     for (const auto &q : parts)
         PSGLD_CK(c, cudaMemcpy2D(q.dst, pitch, q.src, row, row, (size_t)q.rows, cudaMemcpyHostToDevice));
+    // a copy from pageable memory returns with its last part on the way; a
+    // read-back or a sweep on a non-blocking stream would not wait for it
+    PSGLD_CK(c, cudaStreamSynchronize(nullptr));
     c->t_dev_is = -1;
     c->t_done = t;
     c->sweeps_done = sweeps;
