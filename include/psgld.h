@@ -365,7 +365,11 @@ PSGLD_API int64_t psgld_iterations_done(const psgld_ctx *ctx);
 /* Device bytes a context holds once its data is set (psgld_create plus
  * psgld_set_data_*; scratch that those calls free before returning is not
  * counted), for a scheduler that admits work against a memory budget.
- * nnz: observed entries (ignored when dense_path > 0, where V is I x J).
+ * nnz: observed entries (ignored when dense_path > 0, where V is I x J); for
+ * sparse data the bytes are an upper bound whichever parts the entries fall
+ * into.  Not counted: the BF16 copies of gather_bf16, and that entries set on
+ * a context which held more keep its layout's memory when they fill at least
+ * half of it.
  * -1 on invalid sizes.  Needs no GPU. */
 PSGLD_API int64_t psgld_estimate_device_bytes(int64_t I, int64_t J, int32_t K, int32_t B,
                                               int64_t nnz, int32_t dense_path,

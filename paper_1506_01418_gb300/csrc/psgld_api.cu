@@ -14,6 +14,7 @@
 #include <new>
 
 #include "psgld_context.cuh"
+#include "psgld_slots.cuh"
 
 namespace psgld {
 
@@ -1132,17 +1133,20 @@ int64_t psgld_estimate_device_bytes(int64_t I, int64_t J, int32_t K, int32_t B, 
     bytes += 2 * (I + J) * ldk * 4 + (I + J) * ldk * 4 + 2 * (I + J) * ldk * 8 + reduce_blocks() * 8 + 64;
     if (dense_path == 0) {
         // the two part-major entry layouts, the A side's row of each entry,
-        // the lists of the rows with many entries and their chunks' sums
+        // the lists of the rows with many entries and their chunks' sums (the
+        // part with the most may hold every entry)
         for (int side = 0; side < 2; ++side) {
             const int64_t n_rows = side == 0 ? I : J;
             bytes += (B * n_rows + 1) * 4 + nnz * (side == 0 ? 12 : 8) +
-                     16 * (std::min(nnz / (light_row_for(I + J) + 1), B * n_rows) + max_chunks(nnz)) + (4 * ldk + 4) * std::min(max_chunks(nnz), max_chunks(cdiv(nnz, B)) + n_rows);
+                     16 * (std::min(nnz / (light_row_for(I + J) + 1), B * n_rows) + max_chunks(nnz)) +
+                     (4 * ldk + 4) * (nnz / kChunk + std::min(nnz / kMidRow, n_rows));
         }
         // by units of entries: the B side's rows too, and the units' sums
         const int ng = (K + 3) / 4;
         if (step_by_units(I, J, ng, nnz, B))
-            bytes += nnz * 4 + 4 * (cdiv(cdiv(nnz, B), unit_entries(ng)) + 1) * ldk * 4;
-        return bytes;
+            bytes += nnz * 4 + 2 * slot_floats(nnz, unit_entries(ng), (int32_t)ldk) * 4;
+        // up to 256 bytes of rounding for each of the layout's arrays
+        return bytes + 20 * 256;
     }
     bytes += I * J * 4;   // the FP32 copy of V
     const int64_t maxI = cdiv(I, B), maxJ = cdiv(J, B);
