@@ -500,6 +500,11 @@ psgld_status build_layout(psgld_ctx *c, int64_t nnz, const int32_t *i_dev, const
         kept = nullptr;
     }
     void *scratch_mem = dev_alloc(c, scratch.bytes, st);
+    if (!scratch_mem && kept) {   // as large as twice this layout: make room
+        dev_free(c, kept, st);
+        kept = nullptr;
+        scratch_mem = dev_alloc(c, scratch.bytes, st);
+    }
     c->layout_mem = kept ? kept : dev_alloc(c, keep.bytes, st);
     c->layout_bytes = kept ? kept_bytes : keep.bytes;
     auto cleanup = [&]() {

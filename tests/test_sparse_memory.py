@@ -1,6 +1,7 @@
 """Device memory of sparse contexts: psgld_estimate_device_bytes bounds what a
 context holds however its entries fall into parts and whichever form its
-part-step takes."""
+part-step takes, and a load that finds no room beside the layout memory kept
+from the load before gives that back and goes on."""
 import numpy as np
 import pytest
 
@@ -82,3 +83,38 @@ def test_estimate_bounds_what_a_sparse_context_holds(counter, I, J, K, B, n, dia
     assert held <= est
     if diagonal:
         assert est <= 1.5 * held       # and is not far above it where one part has them all
+
+
+@pytest.mark.gpu
+def test_load_goes_on_without_the_kept_layout(counter):
+    I, J, K, B = 4000, 3000, 4, 4
+    many, few = _cells(I, J, B, 400000, 1, False), _cells(I, J, B, 220000, 2, False)
+
+    def load(*sets, limit=None):
+        ch = P.PSGLD(I, J, K, B, 0.0, 1.0, prior_kind=P.PSGLD_PRIOR_GAUSSIAN)
+        for s in sets[:-1]:
+            ch.set_data_coo(*s)
+        counter.limit, counter.refused = limit, 0
+        try:
+            ch.set_data_coo(*sets[-1])
+            return counter.held(), counter.refused
+        finally:
+            counter.limit = None
+            ch.close()
+
+    alone, _ = load(few)
+    kept, _ = load(many, few)
+    assert alone < kept                        # the larger layout's memory stayed
+    # the entries' copies (12 bytes each) and the sort's scratch (24 and its
+    # counts) fit beside this load's own layout, but not beside the kept one
+    lo, hi = alone, 2 * kept + 100 * len(few[0])
+    while hi - lo > 4096:                      # the least limit a load alone needs
+        mid = (lo + hi) // 2
+        try:
+            load(few, limit=mid)
+            hi = mid
+        except P.PsgldError as e:
+            assert e.status == P.PSGLD_ERR_OOM
+            lo = mid
+    held, refused = load(many, few, limit=hi)
+    assert refused > 0 and held <= hi
