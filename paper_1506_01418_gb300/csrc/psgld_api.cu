@@ -1143,7 +1143,7 @@ int64_t psgld_estimate_device_bytes(int64_t I, int64_t J, int32_t K, int32_t B, 
         }
         // by units of entries: the B side's rows too, and the units' sums
         const int ng = (K + 3) / 4;
-        if (step_by_units(I, J, ng, nnz, B))
+        if (step_by_units(I, J, ng, nnz, B, false) || step_by_units(I, J, ng, nnz, B, true))
             bytes += nnz * 4 + 2 * slot_floats(nnz, unit_entries(ng), (int32_t)ldk) * 4;
         // up to 256 bytes of rounding for each of the layout's arrays
         return bytes + 20 * 256;

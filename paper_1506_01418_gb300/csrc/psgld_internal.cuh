@@ -260,7 +260,7 @@ psgld_status launch_part_step(psgld_ctx *c, int64_t t, const int64_t *t_dev,
 psgld_status launch_rows(psgld_ctx *c, int part, int64_t t, const int64_t *t_dev, int64_t t_add, cudaStream_t st);
 // The same by units of consecutive entries (psgld_units.cu): whether a part
 // of nnz / B entries of I x J takes that form.
-bool step_by_units(int64_t I, int64_t J, int ngroups, int64_t nnz, int B);
+bool step_by_units(int64_t I, int64_t J, int ngroups, int64_t nnz, int B, bool bf16);
 int unit_entries(int ngroups);
 int rows_groups(int ngroups);   // float4 groups, with padding, of a row in psgld_rows.cu
 psgld_status prepare_units(psgld_ctx *c);
@@ -271,6 +271,7 @@ psgld_status launch_units(psgld_ctx *c, int part, int64_t t, const int64_t *t_de
 // ldk rounded up to 8) and writes those of the new ones; built from the
 // current factors by build_gather_shadows (allocating them).
 bool gather_bf16(const psgld_ctx *c);
+int gather_ld16(int ldk);   // their rows: ldk rounded up to 8 (16 bytes)
 psgld_status build_gather_shadows(psgld_ctx *c, cudaStream_t st);
 
 // After a synchronisation point: PSGLD_ERR_TIMEOUT (and the flag cleared) if

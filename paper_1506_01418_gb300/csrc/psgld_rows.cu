@@ -601,10 +601,9 @@ __global__ void gather_copy_kernel(const float *__restrict__ X, int64_t n, int l
     }
 }
 
-// rows of the BF16 copies: ldk rounded up to 8 (16 bytes)
-int ld16_for(int ldk) { return 8 * ((ldk + 7) / 8); }
-
 }  // namespace
+
+int gather_ld16(int ldk) { return 8 * ((ldk + 7) / 8); }
 
 int rows_groups(int ng) { return pick_rows<false>(ng).groups; }
 
@@ -613,7 +612,7 @@ bool gather_bf16(const psgld_ctx *c) { return c->opt.gather_bf16 && !c->dense &&
 psgld_status build_gather_shadows(psgld_ctx *c, cudaStream_t st)
 {
     if (!c->opt.gather_bf16 || c->dense || !c->has_factors) return PSGLD_OK;
-    const int ld16 = ld16_for(c->ldk);
+    const int ld16 = gather_ld16(c->ldk);
     for (int side = 0; side < 2; ++side) {
         const int64_t n = side == 0 ? c->I : c->J;
         const float *X = side == 0 ? c->W[c->wcur] : c->Ht[c->hcur];
@@ -686,7 +685,7 @@ psgld_status launch_rows(psgld_ctx *c, int part, int64_t t, const int64_t *t_dev
     const int64_t grid = (int64_t)P.side[0].n_heavy + P.side[1].n_heavy + mid + light;
     P.K = c->K;
     P.ldk = c->ldk;
-    P.ld16 = ld16_for(c->ldk);
+    P.ld16 = gather_ld16(c->ldk);
     P.ng = c->ngroups;
     P.phi_inv = (float)(1.0 / c->phi);
     P.p = (float)c->p;

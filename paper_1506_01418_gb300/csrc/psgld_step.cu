@@ -250,8 +250,7 @@ psgld_status launch_part_step(psgld_ctx *c, int64_t t, const int64_t *t_dev, int
         PSGLD_CK(c, cudaEventRecordWithFlags(c->ev_start[part], st, rec_flags));
     }
     if (!c->dense) {
-        // (the BF16 copies are written by the rows form alone)
-        if (c->units && !gather_bf16(c)) {
+        if (c->units) {
             const psgld_status rs = launch_units(c, part, t, t_dev, t_add, st, prof ? c->ev_mid[part] : nullptr, rec_flags);
             if (rs != PSGLD_OK) return rs;
         } else {

@@ -49,12 +49,14 @@ struct GradSide {
     int64_t base;          // first entry of the part
     int64_t n;             // entries of the part
     int64_t units;         // ceil(n / E)
+    const uint16_t *Y16;   // BF16 copy of Y_cur (rows of ld16), gathered instead of it
     int prefetch_own;      // 1: own rows go to L2 with the gathers (own factor beyond L2)
 };
 
 struct GradParams {
     GradSide side[2];
     int ldk, lds, ngroups;    // row length, shared-memory row stride (floats), float4 groups
+    int ld16, lds16;          // BF16 gathers: row length and shared-memory row stride (elements)
     float phi_inv, p, mu_min;
     int p_mode;               // 0: p = 0, 1: p = 1, 2: p = 2, 3: other
     int *err;                 // set to 16 when a bulk copy wait runs out
@@ -69,13 +71,14 @@ struct UpdSide {
     const float *partial;     // head / tail partial sums of the gradient kernel
     int64_t base;             // first entry of the part
     int64_t items;            // n_rows * ngroups (0 when the factor is frozen)
+    uint16_t *X16_next;       // BF16 copy of X_next (rows of ld16)
     float prior_a, prior_b;   // d log p(x)/dx = prior_a + prior_b * x
 };
 
 struct UpdParams {
     UpdSide side[2];
     StepNoise noise;
-    int K, ldk, ngroups, unit_shift;
+    int K, ldk, ld16, ngroups, unit_shift;
     uint32_t div_magic;       // ceil(2^32 / ngroups) when item * ngroups < 2^32, else 0
 };
 
@@ -166,10 +169,18 @@ __device__ __forceinline__ void prefetch_l2(const void *src, uint32_t bytes)
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" :: "l"(src), "r"(bytes) : "memory");
 }
 
-// q-th float4 group of row `row` of the warp's gathered rows.
-__device__ __forceinline__ float4 ys4(const float *ys, int row, int q, int lds)
+// q-th float4 group of row `row` of the warp's gathered rows: FP32 rows of
+// `stride` floats, or (BF) BF16 rows of `stride` elements.
+template <bool BF>
+__device__ __forceinline__ float4 ys4(const float *ys, int row, int q, int stride)
 {
-    return *reinterpret_cast<const float4 *>(ys + (size_t)row * lds + 4 * q);
+    if constexpr (BF) {
+        const uint2 v = *reinterpret_cast<const uint2 *>(reinterpret_cast<const uint16_t *>(ys) + (size_t)row * stride + 4 * q);
+        return make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xFFFF0000u),
+                           __uint_as_float(v.y << 16), __uint_as_float(v.y & 0xFFFF0000u));
+    } else {
+        return *reinterpret_cast<const float4 *>(ys + (size_t)row * stride + 4 * q);
+    }
 }
 
 // A unit's entries as each lane loads them, one unit ahead of its work:
@@ -201,16 +212,17 @@ __device__ __forceinline__ UnitIn load_unit(const GradParams &P, int64_t u)
 
 // One unit (E consecutive entries of side SID's part order) on one warp; SID
 // is a template parameter so that the side's fields are fixed parameter
-// offsets.  `bar` completes once per unit, phase
+// offsets.  BF: the gathered rows are the BF16 copies (half the bytes;
+// products and sums stay FP32).  `bar` completes once per unit, phase
 // `parity`.  False when the gathers did not land in time (the warp stops).
-template <int SID, int S, int NG, int E>
+template <int SID, int S, int NG, int E, bool BF>
 __device__ __forceinline__ bool grad_unit(const GradParams &P, int64_t u, const UnitIn &in, float *ys,
                                           float *es, int *ow, int *sg, uint64_t *bar, uint32_t parity)
 {
     constexpr int R = 32 / S;      // sub-teams per warp
     constexpr int NGP = S * NG;    // float4 groups a sub-team covers (>= ngroups)
     const int lane32 = threadIdx.x & 31;
-    const int ng = P.ngroups, ldk = P.ldk, lds = P.lds;
+    const int ng = P.ngroups, ldk = P.ldk, lds = BF ? P.lds16 : P.lds;
     const GradSide &Sd = P.side[SID];
     const int n = (int)(Sd.n - u * E < E ? Sd.n - u * E : E);
 
@@ -220,7 +232,7 @@ __device__ __forceinline__ bool grad_unit(const GradParams &P, int64_t u, const 
     const float vv = in.vv;
     const int prev_own = __shfl_sync(0xffffffffu, in.edge, 0);   // rows of the entries just outside the unit
     const int next_own = __shfl_sync(0xffffffffu, in.edge, 1);
-    const uint32_t row_bytes = (uint32_t)ldk * 4u;
+    const uint32_t row_bytes = BF ? (uint32_t)P.ld16 * 2u : (uint32_t)ldk * 4u;
 
     // ---- 2. bulk gathers into shared memory, once every lane is done with
     // the previous unit's (its reads ordered before the copies' writes)
@@ -234,7 +246,12 @@ __device__ __forceinline__ bool grad_unit(const GradParams &P, int64_t u, const 
         // before the copies are issued -- so the wait surely runs out
         for (uint32_t it = 0; it < P.wait_polls && !done; ++it) done = mbar_test_wait(bar, parity);
     }
-    if (valid) bulk_g2s(ys + (size_t)lane32 * lds, Sd.Y_cur + (int64_t)jj * ldk, row_bytes, bar);
+    if (valid) {
+        if constexpr (BF)
+            bulk_g2s(reinterpret_cast<uint16_t *>(ys) + (size_t)lane32 * lds, Sd.Y16 + (int64_t)jj * P.ld16, row_bytes, bar);
+        else
+            bulk_g2s(ys + (size_t)lane32 * lds, Sd.Y_cur + (int64_t)jj * ldk, row_bytes, bar);
+    }
     // each row segment's own row on its way to L2 while the gathers land
     const int own_prev_lane = __shfl_up_sync(0xffffffffu, own, 1);
     const bool seg_start = valid && (lane32 == 0 || own != own_prev_lane);
@@ -268,7 +285,7 @@ __device__ __forceinline__ bool grad_unit(const GradParams &P, int64_t u, const 
         float d = 0.f;
 #pragma unroll
         for (int q = 0; q < NGP; ++q)
-            if (q < ng) d = dot4(q < XP ? xp[q < XP ? q : 0] : ldg4(x + 4 * q), ys4(ys, lane32, q, lds), d);
+            if (q < ng) d = dot4(q < XP ? xp[q < XP ? q : 0] : ldg4(x + 4 * q), ys4<BF>(ys, lane32, q, lds), d);
         e = tweedie_e(P, vv, d);
     }
     const unsigned smask = __ballot_sync(0xffffffffu, seg_start);
@@ -295,7 +312,7 @@ __device__ __forceinline__ bool grad_unit(const GradParams &P, int64_t u, const 
 #pragma unroll
             for (int g = 0; g < NG; ++g) {
                 const int q = lane + g * S;
-                if (q < ng) axpy4(acc[g], es_, ys4(ys, sl, q, lds));
+                if (q < ng) axpy4(acc[g], es_, ys4<BF>(ys, sl, q, lds));
             }
         }
 #pragma unroll
@@ -331,7 +348,7 @@ __device__ __forceinline__ bool grad_unit(const GradParams &P, int64_t u, const 
 #pragma unroll
                 for (int g = 0; g < NG; ++g) {
                     const int q = lane + g * S;
-                    if (q < ng) axpy4(acc[g], es_, ys4(ys, sl, q, lds));
+                    if (q < ng) axpy4(acc[g], es_, ys4<BF>(ys, sl, q, lds));
                 }
             }
             float *dst = (k == 0 && prev_own == row) ? Sd.partial + head_slot(u, ldk)
@@ -351,7 +368,7 @@ __device__ __forceinline__ bool grad_unit(const GradParams &P, int64_t u, const 
 // grid of one CTA per 4 units gives every warp one unit; a smaller grid
 // keeps warps resident over several), loading the next unit's entries
 // before working on the current one.
-template <int S, int NG, int E>
+template <int S, int NG, int E, bool BF>
 __global__ void __launch_bounds__(kGradThreads) grad_kernel(const __grid_constant__ GradParams P)
 {
     extern __shared__ float4 smem4[];
@@ -376,8 +393,8 @@ __global__ void __launch_bounds__(kGradThreads) grad_kernel(const __grid_constan
         const int64_t nu = u + T;
         UnitIn nxt{-1, 0, 0.f, -1};
         if (nu < U) nxt = nu < U0 ? load_unit<0, E>(P, nu) : load_unit<1, E>(P, nu - U0);
-        const bool ok = u < U0 ? grad_unit<0, S, NG, E>(P, u, cur, ys, es, ow, sg, bar, parity)
-                               : grad_unit<1, S, NG, E>(P, u - U0, cur, ys, es, ow, sg, bar, parity);
+        const bool ok = u < U0 ? grad_unit<0, S, NG, E, BF>(P, u, cur, ys, es, ow, sg, bar, parity)
+                               : grad_unit<1, S, NG, E, BF>(P, u - U0, cur, ys, es, ow, sg, bar, parity);
         if (!ok) return;
         cur = nxt;
     }
@@ -385,7 +402,7 @@ __global__ void __launch_bounds__(kGradThreads) grad_kernel(const __grid_constan
 
 // One (row, float4 group) item of factor SID (0 = W, 1 = H^T): items and
 // factor offsets in 32 bits (step_by_units checks the sizes), slots in 64.
-template <int SID>
+template <int SID, bool BF>
 __device__ __forceinline__ void update_item32(const UpdParams &P, uint32_t item, float eps, float sd,
                                               uint32_t t_lo, uint32_t t_hi)
 {
@@ -422,8 +439,14 @@ __device__ __forceinline__ void update_item32(const UpdParams &P, uint32_t item,
     float4 o = dev::langevin4(P.noise, Sd.prior_a, Sd.prior_b, x, g, z, eps, sd);
     dev::mask_padding(o, q, (uint32_t)P.K);
     *reinterpret_cast<float4 *>(Sd.X_next + off) = o;
+    if constexpr (BF) {
+        const __nv_bfloat162 a = __floats2bfloat162_rn(o.x, o.y), b = __floats2bfloat162_rn(o.z, o.w);
+        *reinterpret_cast<uint2 *>(Sd.X16_next + (int64_t)row * P.ld16 + 4u * q) =
+            make_uint2(*reinterpret_cast<const uint32_t *>(&a), *reinterpret_cast<const uint32_t *>(&b));
+    }
 }
 
+template <bool BF>
 __global__ void __launch_bounds__(kThreads, 5) units_update_kernel(const __grid_constant__ UpdParams P)
 {
     const StepNoise &N = P.noise;
@@ -438,8 +461,8 @@ __global__ void __launch_bounds__(kThreads, 5) units_update_kernel(const __grid_
     const uint32_t n0 = (uint32_t)P.side[0].items, n1 = (uint32_t)P.side[1].items;
     const uint32_t stride = gridDim.x * kThreads;
     uint32_t a = blockIdx.x * kThreads + threadIdx.x;
-    for (; a < n0; a += stride) update_item32<0>(P, a, eps, sd, t_lo, t_hi);
-    for (a -= n0; a < n1; a += stride) update_item32<1>(P, a, eps, sd, t_lo, t_hi);
+    for (; a < n0; a += stride) update_item32<0, BF>(P, a, eps, sd, t_lo, t_hi);
+    for (a -= n0; a < n1; a += stride) update_item32<1, BF>(P, a, eps, sd, t_lo, t_hi);
 }
 
 using GradFn = void (*)(GradParams);
@@ -469,30 +492,42 @@ Shape shape_for(int ngroups)
     return sh;
 }
 
-GradFn pick_grad(const Shape &sh)
+template <bool BF>
+GradFn pick_grad_t(const Shape &sh)
 {
     if (sh.NG == 1) {
         switch (sh.S) {
-        case 1: return grad_kernel<1, 1, 32>;
-        case 2: return grad_kernel<2, 1, 32>;
-        case 4: return grad_kernel<4, 1, 32>;
+        case 1: return grad_kernel<1, 1, 32, BF>;
+        case 2: return grad_kernel<2, 1, 32, BF>;
+        case 4: return grad_kernel<4, 1, 32, BF>;
         }
     }
     if (sh.NG == 2) {
         switch (sh.S) {
-        case 4: return grad_kernel<4, 2, 32>;
-        case 8: return grad_kernel<8, 2, 32>;
-        case 16: return grad_kernel<16, 2, 32>;
-        case 32: return grad_kernel<32, 2, 16>;
+        case 4: return grad_kernel<4, 2, 32, BF>;
+        case 8: return grad_kernel<8, 2, 32, BF>;
+        case 16: return grad_kernel<16, 2, 32, BF>;
+        case 32: return grad_kernel<32, 2, 16, BF>;
         }
     }
     if (sh.S == 32) {
         switch (sh.NG) {
-        case 3: return grad_kernel<32, 3, 8>;
-        case 4: return grad_kernel<32, 4, 8>;
+        case 3: return grad_kernel<32, 3, 8, BF>;
+        case 4: return grad_kernel<32, 4, 8, BF>;
         }
     }
     return nullptr;
+}
+
+// bf: the variant that gathers the BF16 copies of the factors
+GradFn pick_grad(const Shape &sh, bool bf) { return bf ? pick_grad_t<true>(sh) : pick_grad_t<false>(sh); }
+
+// Shared-memory stride of the BF16 rows: lds16 / 8 odd, so that the lanes'
+// 8-byte reads of distinct rows spread over the banks.
+int lds16_for(int ldk)
+{
+    const int m = gather_ld16(ldk) / 8;
+    return 8 * ((m & 1) ? m : m + 1);
 }
 
 size_t grad_smem(const Shape &sh)
@@ -520,15 +555,25 @@ int unit_entries(int ngroups) { return shape_for(ngroups).E; }
 //   K = 128, 200: 49 / 66, 81 / 115; 35 000 rows, 31 000 entries, 429 / 455,
 //   584 / 763; 28 000 rows, 62 000 entries, 487 / 457, 715 / 784;
 //   K = 300: 25 000 entries 137 / 123, 2500 59 / 117.
+// With BF16 gathers the rows' gathers cost half as much and the flat update
+// pays on the largest factors alone: 3.05 10^5 rows, rho 0.4, K = 16, 20, 50,
+// 96: 373 / 518, 448 / 906, 1039 / 1624, 1697 / 2088; rho 1.5 525 / 430,
+// 683 / 784, 1490 / 1271, 2328 / 1755; 4.98 10^5 rows, rho 1.0, K = 16, 72:
+// 2614 / 4169, 10007 / 11659; and where 5 or 6 of a row's 8 lanes work:
+// 8 10^4 rows, rho 0.8, K = 20: 408 / 455; 10^5 rows, rho 0.4: 119 / 143.
 // Items and factor offsets in 32 bits.
-bool step_by_units(int64_t I, int64_t J, int ngroups, int64_t nnz, int B)
+bool step_by_units(int64_t I, int64_t J, int ngroups, int64_t nnz, int B, bool bf16)
 {
     const int64_t rows = I + J, items = rows * ngroups, lim = (1ll << 31) - 1;
     if (items > lim || std::max(I, J) * 4 * ngroups > lim) return false;
-    if (ngroups > 24 && nnz < (ngroups <= 64 ? 1536ll : 128ll) * ngroups * B) return true;
-    if (ngroups <= 2 || items <= (1 << 19)) return false;
     const double padding = (double)rows_groups(ngroups) / ngroups - 1.0;
     const double rho = 2.0 * (double)nnz / ((double)B * (double)rows);
+    if (bf16) {
+        if (rows > 1 << 18 && ngroups < 32 && rho < (ngroups <= 16 ? 2.4e-6 : 1.8e-6) * (double)rows + padding) return true;
+        return (ngroups == 5 || ngroups == 6) && rows > 1 << 16 && rho < 2.0;
+    }
+    if (ngroups > 24 && nnz < (ngroups <= 64 ? 1536ll : 128ll) * ngroups * B) return true;
+    if (ngroups <= 2 || items <= (1 << 19)) return false;
     return rho < (ngroups <= 16 ? 2.0 : 1.0) + 4.0 * padding;
 }
 
@@ -564,9 +609,11 @@ static int64_t resident_wave(const void *f, int threads, size_t smem)
 psgld_status prepare_units(psgld_ctx *c)
 {
     const Shape sh = shape_for(c->ngroups);
-    const GradFn fn = pick_grad(sh);
-    if (!fn) return fail(c, PSGLD_ERR_ARG, "unsupported K");
-    PSGLD_CK(c, cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)grad_smem(sh)));
+    for (int bf = 0; bf < 2; ++bf) {
+        const GradFn fn = pick_grad(sh, bf != 0);
+        if (!fn) return fail(c, PSGLD_ERR_ARG, "unsupported K");
+        PSGLD_CK(c, cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)grad_smem(sh)));
+    }
     return side_stream(c);
 }
 
@@ -574,7 +621,8 @@ psgld_status launch_units(psgld_ctx *c, int part, int64_t t, const int64_t *t_de
                           cudaEvent_t mid, unsigned rec_flags)
 {
     const Shape sh = shape_for(c->ngroups);
-    const GradFn fn = pick_grad(sh);
+    const bool bf = gather_bf16(c);
+    const GradFn fn = pick_grad(sh, bf);
     const bool upd[2] = {!c->opt.freeze_W, !c->opt.freeze_H};
     GradParams GP{};
     UpdParams UP{};
@@ -594,6 +642,10 @@ psgld_status launch_units(psgld_ctx *c, int part, int64_t t, const int64_t *t_de
         Gs.base = base;
         Gs.n = n;
         Gs.units = upd[s] ? (n + sh.E - 1) / sh.E : 0;
+        if (bf) {
+            Gs.Y16 = s == 0 ? c->H16[c->hcur] : c->W16[c->wcur];
+            Us.X16_next = s == 0 ? c->W16[c->wcur ^ 1] : c->H16[c->hcur ^ 1];
+        }
         Gs.prefetch_own = 4.0 * (double)n_rows * c->ldk > 64.0 * (1 << 20);
         Us.X_cur = Gs.X_cur;
         Us.X_next = s == 0 ? c->W[c->wcur ^ 1] : c->Ht[c->hcur ^ 1];
@@ -611,6 +663,8 @@ psgld_status launch_units(psgld_ctx *c, int part, int64_t t, const int64_t *t_de
     }
     GP.ldk = c->ldk;
     GP.lds = sh.lds;
+    GP.ld16 = gather_ld16(c->ldk);
+    GP.lds16 = lds16_for(c->ldk);
     GP.ngroups = c->ngroups;
     GP.phi_inv = (float)(1.0 / c->phi);
     GP.p = (float)c->p;
@@ -621,6 +675,7 @@ psgld_status launch_units(psgld_ctx *c, int part, int64_t t, const int64_t *t_de
     fill_noise(c, part, t, t_dev, t_add, UP.noise);
     UP.K = c->K;
     UP.ldk = c->ldk;
+    UP.ld16 = GP.ld16;
     UP.ngroups = c->ngroups;
     UP.unit_shift = sh.E == 32 ? 5 : sh.E == 16 ? 4 : 3;
     const int64_t max_items = std::max(UP.side[0].items, UP.side[1].items);
@@ -631,7 +686,7 @@ psgld_status launch_units(psgld_ctx *c, int part, int64_t t, const int64_t *t_de
         if (side < 2) U.side[side ^ 1].items = 0;
         const int64_t n = U.side[0].items + U.side[1].items;
         const int grid = (int)std::min<int64_t>((n + kThreads - 1) / kThreads, 152 * 16);
-        if (grid > 0) units_update_kernel<<<grid, kThreads, 0, ss>>>(U);
+        if (grid > 0) (bf ? units_update_kernel<true> : units_update_kernel<false>)<<<grid, kThreads, 0, ss>>>(U);
     };
     // resident: one wave of CTAs whose warps walk several units each (the
     // next unit's entries load during the current one); otherwise one unit
