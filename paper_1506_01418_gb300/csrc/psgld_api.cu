@@ -1138,12 +1138,13 @@ int64_t psgld_estimate_device_bytes(int64_t I, int64_t J, int32_t K, int32_t B, 
         for (int side = 0; side < 2; ++side) {
             const int64_t n_rows = side == 0 ? I : J;
             bytes += (B * n_rows + 1) * 4 + nnz * (side == 0 ? 12 : 8) +
-                     16 * (std::min(nnz / (light_row_for(I + J) + 1), B * n_rows) + max_chunks(nnz)) +
+                     16 * (std::min(nnz / (light_row_for(I, J, (int)(ldk / 4)) + 1), B * n_rows) + max_chunks(nnz)) +
                      (4 * ldk + 4) * (nnz / kChunk + std::min(nnz / kMidRow, n_rows));
         }
         // by units of entries: the B side's rows too, and the units' sums
+        // (with gather_bf16 only some of these contexts)
         const int ng = (K + 3) / 4;
-        if (step_by_units(I, J, ng, nnz, B, false) || step_by_units(I, J, ng, nnz, B, true))
+        if (step_by_units(I, J, ng, nnz, B, false))
             bytes += nnz * 4 + 2 * slot_floats(nnz, unit_entries(ng), (int32_t)ldk) * 4;
         // up to 256 bytes of rounding for each of the layout's arrays
         return bytes + 20 * 256;

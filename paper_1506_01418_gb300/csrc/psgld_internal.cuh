@@ -61,8 +61,14 @@ struct SideLayout {
 // (psgld_rows.cu); above, a block takes each kChunk.
 constexpr uint32_t kMidRow = 128, kChunk = 512;
 // ... and up to which one of a warp's teams of lanes does: few when the rows
-// of a part do not fill the chip's warps anyway.
-constexpr int light_row_for(int64_t rows) { return rows < 152 * 32 ? 2 : 16; }
+// of a part do not fill the chip's warps anyway, fewer where a team is one
+// lane, which walks its entries one after the other, and one side has few
+// rows, hence many entries in each: 10^5 x 5000, K = 4, B = 8, 0.4 and 0.6 10^6
+// entries: 78 and 90 us a sweep with 16, 69 and 68 with 8.
+constexpr int light_row_for(int64_t I, int64_t J, int ngroups)
+{
+    return I + J < 152 * 32 ? 2 : ngroups == 1 && (I < J ? I : J) < 152 * 64 ? 8 : 16;
+}
 // chunks of rows with more than kMidRow entries, at most, among n entries
 constexpr int64_t max_chunks(int64_t n) { return n / kChunk + n / kMidRow; }
 

@@ -461,7 +461,7 @@ psgld_status build_layout(psgld_ctx *c, int64_t nnz, const int32_t *i_dev, const
     free_layout(c);
     const int64_t I = c->I, J = c->J, n = nnz;
     const int B = c->B;
-    c->light_row = light_row_for(I + J);
+    c->light_row = light_row_for(I, J, c->ngroups);
     c->units = step_by_units(I, J, c->ngroups, n, B, c->opt.gather_bf16 != 0);
     if (c->units) {
         const psgld_status s = prepare_units(c);

@@ -549,7 +549,13 @@ int unit_entries(int ngroups) { return shape_for(ngroups).E; }
 //   2933 / 2667; 2.5 10^5 rows, rho 3.2, K = 20, 32, 72, 96: 2112 / 2575,
 //   2535 / 2629, 5405 / 5595, 6470 / 5679; 8 10^4 rows, rho 3.9, K = 36:
 //   811 / 886, K = 64: 1119 / 965; 5.5 10^4 rows, rho 14.5, K = 72:
-//   1242 / 1157.  Up to K = 8 a row is one or two lanes and rows as fast.
+//   1242 / 1157.  Up to K = 8 a row is one or two lanes: rows as fast, but for
+//   the largest factors: 3.05 10^5 rows, rho 0.5, K = 4: 192 / 232; 4.98 10^5
+//   rows, rho 0.5, K = 8: 1358 / 1703.  Smaller factors where padding counts:
+//   8 10^4 rows, rho 1.0, K = 20: 382 / 446, K = 36: rho 0.5 605 / 581, rho 4
+//   828 / 910; 3.5 10^4 rows, K = 36, rho 4: 117 / 134.  Beyond K = 64 padding
+//   counts for less: 1.5 10^5 rows, rho 2, K = 100, 200: 1421 / 1195,
+//   2605 / 2027.
 //   K > 96 and few entries in a part, where a launch is as long as one
 //   warp's walk over a row with a hundred entries.  1600 rows, 25 000 entries,
 //   K = 128, 200: 49 / 66, 81 / 115; 35 000 rows, 31 000 entries, 429 / 455,
@@ -568,13 +574,13 @@ bool step_by_units(int64_t I, int64_t J, int ngroups, int64_t nnz, int B, bool b
     if (items > lim || std::max(I, J) * 4 * ngroups > lim) return false;
     const double padding = (double)rows_groups(ngroups) / ngroups - 1.0;
     const double rho = 2.0 * (double)nnz / ((double)B * (double)rows);
-    if (bf16) {
-        if (rows > 1 << 18 && ngroups < 32 && rho < (ngroups <= 16 ? 2.4e-6 : 1.8e-6) * (double)rows + padding) return true;
-        return (ngroups == 5 || ngroups == 6) && rows > 1 << 16 && rho < 2.0;
-    }
+    if (rows > 1 << 18 && ngroups < 32 && rho < (ngroups <= 16 ? 2.4e-6 : 1.8e-6) * (double)rows + padding) return true;
+    if ((ngroups == 5 || ngroups == 6) && rows > 1 << 16 && rho < 2.0) return true;
+    if (bf16) return false;
+    if (ngroups == 9 && rows > 1 << 15 && rho >= 2.0 && rho < 6.0) return true;
     if (ngroups > 24 && nnz < (ngroups <= 64 ? 1536ll : 128ll) * ngroups * B) return true;
     if (ngroups <= 2 || items <= (1 << 19)) return false;
-    return rho < (ngroups <= 16 ? 2.0 : 1.0) + 4.0 * padding;
+    return rho < (ngroups <= 16 ? 2.0 + 4.0 * padding : 1.0 + 2.0 * padding);
 }
 
 // CTAs of kernel `f` (`threads` threads, `smem` bytes of dynamic shared
