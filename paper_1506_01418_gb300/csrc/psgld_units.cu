@@ -553,8 +553,8 @@ int unit_entries(int ngroups) { return shape_for(ngroups).E; }
 //   the largest factors: 3.05 10^5 rows, rho 0.5, K = 4: 192 / 232; 4.98 10^5
 //   rows, rho 0.5, K = 8: 1358 / 1703.  Smaller factors where padding counts:
 //   8 10^4 rows, rho 1.0, K = 20: 382 / 446, K = 36: rho 0.5 605 / 581, rho 4
-//   828 / 910; 3.5 10^4 rows, K = 36, rho 4: 117 / 134.  Beyond K = 64 padding
-//   counts for less: 1.5 10^5 rows, rho 2, K = 100, 200: 1421 / 1195,
+//   828 / 910; 3.5 10^4 rows, K = 36, rho 4: 117 / 134.  From K = 65 to 256
+//   padding counts for less: 1.5 10^5 rows, rho 2, K = 100, 200: 1421 / 1195,
 //   2605 / 2027.
 //   K > 96 and few entries in a part, where a launch is as long as one
 //   warp's walk over a row with a hundred entries.  1600 rows, 25 000 entries,
@@ -580,7 +580,7 @@ bool step_by_units(int64_t I, int64_t J, int ngroups, int64_t nnz, int B, bool b
     if (ngroups == 9 && rows > 1 << 15 && rho >= 2.0 && rho < 6.0) return true;
     if (ngroups > 24 && nnz < (ngroups <= 64 ? 1536ll : 128ll) * ngroups * B) return true;
     if (ngroups <= 2 || items <= (1 << 19)) return false;
-    return rho < (ngroups <= 16 ? 2.0 + 4.0 * padding : 1.0 + 2.0 * padding);
+    return rho < (ngroups <= 16 ? 2.0 : 1.0) + (ngroups <= 16 || ngroups > 64 ? 4.0 : 2.0) * padding;
 }
 
 // CTAs of kernel `f` (`threads` threads, `smem` bytes of dynamic shared
