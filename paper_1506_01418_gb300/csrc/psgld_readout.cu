@@ -46,11 +46,48 @@ constexpr size_t kHost = 768 << 10;
 constexpr int64_t kPerHelper = 4 << 20;
 constexpr unsigned kThreads = 8;
 
-// One staging area for the process, used by one read-back at a time, given
-// back with the last context.
+// Staging areas of the process, at most kAreas (64 MB), one to a read-back
+// while it lasts, given back with the last context.  A read-back that finds
+// them all taken goes without.
+constexpr int kAreas = 8;
 std::mutex g_stage_mutex;
-char *g_stage = nullptr;
+char *g_free[kAreas];
+int g_n_free = 0, g_areas = 0, g_readers = 0;
 int64_t g_contexts = 0;
+
+class Staging {
+public:
+    // the area, if one is to be had, and how many read-backs there are now
+    char *take(int *readers)
+    {
+        {
+            std::lock_guard<std::mutex> l(g_stage_mutex);
+            *readers = ++g_readers;
+            reading_ = true;
+            if (g_n_free > 0) return area_ = g_free[--g_n_free];
+            if (g_areas == kAreas) return nullptr;
+            ++g_areas;
+        }
+        if (cudaHostAlloc(reinterpret_cast<void **>(&area_), 2 * kHalf, cudaHostAllocPortable) != cudaSuccess) {
+            cudaGetLastError();
+            area_ = nullptr;
+            std::lock_guard<std::mutex> l(g_stage_mutex);
+            --g_areas;
+        }
+        return area_;
+    }
+    ~Staging()
+    {
+        if (!reading_) return;
+        std::lock_guard<std::mutex> l(g_stage_mutex);
+        --g_readers;
+        if (area_) g_free[g_n_free++] = area_;
+    }
+
+private:
+    char *area_ = nullptr;
+    bool reading_ = false;
+};
 
 // Threads that copy slices beside the caller's, for one read-back.
 class Crew {
@@ -173,10 +210,8 @@ void use_staging(int by)
 {
     std::lock_guard<std::mutex> l(g_stage_mutex);
     g_contexts += by;
-    if (g_contexts == 0 && g_stage) {
-        cudaFreeHost(g_stage);
-        g_stage = nullptr;
-    }
+    if (g_contexts > 0) return;
+    for (; g_n_free > 0; --g_areas) cudaFreeHost(g_free[--g_n_free]);
 }
 
 psgld_status read_moments(psgld_ctx *c, double *const (&out)[2][2])
@@ -196,15 +231,10 @@ psgld_status read_moments(psgld_ctx *c, double *const (&out)[2][2])
         }
     cudaStream_t st = c->capture_stream;
     if (total <= (int64_t)kHost) return divide_on_host(c, out, st);
-    std::unique_lock<std::mutex> stage(g_stage_mutex, std::defer_lock);
-    if (total > (int64_t)kDirect) {
-        stage.lock();
-        if (!g_stage && cudaHostAlloc(reinterpret_cast<void **>(&g_stage), 2 * kHalf, cudaHostAllocPortable) != cudaSuccess) {
-            cudaGetLastError();
-            g_stage = nullptr;
-        }
-    }
-    if (!stage.owns_lock() || !g_stage) {
+    Staging staging;
+    int readers = 1;
+    char *const area = total > (int64_t)kDirect ? staging.take(&readers) : nullptr;
+    if (!area) {
         for (const Piece &p : pieces) {
             PSGLD_CK(c, form(c, p, st));
             PSGLD_CK(c, cudaMemcpyAsync(p.out, c->G, row * (size_t)p.rows, cudaMemcpyDefault, st));
@@ -217,12 +247,13 @@ psgld_status read_moments(psgld_ctx *c, double *const (&out)[2][2])
     for (auto &ev : full)
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
     {
-        const unsigned hw = std::max(1u, std::thread::hardware_concurrency());
-        Crew crew((unsigned)std::min<int64_t>(std::min(kThreads, hw) - 1, total / kPerHelper));
+        // the host's cores among the read-backs under way
+        const unsigned mine = std::max(1u, std::thread::hardware_concurrency() / (unsigned)readers);
+        Crew crew((unsigned)std::min<int64_t>(std::min(kThreads, mine) - 1, total / kPerHelper));
         auto fetch = [&](size_t k) {
             e = form(c, pieces[k], st);
             if (e == cudaSuccess)
-                e = cudaMemcpyAsync(g_stage + (k & 1) * kHalf, c->G, row * (size_t)pieces[k].rows, cudaMemcpyDeviceToHost, st);
+                e = cudaMemcpyAsync(area + (k & 1) * kHalf, c->G, row * (size_t)pieces[k].rows, cudaMemcpyDeviceToHost, st);
             if (e == cudaSuccess) e = cudaEventRecord(full[k & 1], st);
         };
         if (e == cudaSuccess) fetch(0);
@@ -230,7 +261,7 @@ psgld_status read_moments(psgld_ctx *c, double *const (&out)[2][2])
             if (k + 1 < pieces.size()) fetch(k + 1);
             if (e == cudaSuccess) e = cudaEventSynchronize(full[k & 1]);
             if (e == cudaSuccess)
-                crew.copy(reinterpret_cast<char *>(pieces[k].out), g_stage + (k & 1) * kHalf, row * (size_t)pieces[k].rows);
+                crew.copy(reinterpret_cast<char *>(pieces[k].out), area + (k & 1) * kHalf, row * (size_t)pieces[k].rows);
         }
     }
     if (e != cudaSuccess) cudaStreamSynchronize(st);   // nothing in flight into the staging area
