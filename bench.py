@@ -520,18 +520,15 @@ def run_ours(args, wl_name, wl):
     else:
         # the part-step's time from the timed sweeps themselves (sweep / B,
         # which also holds 1/B of the posterior accumulation), so that it
-        # never exceeds the sweep it belongs to; the profiled pass only
-        # gives the split between the two kernels
+        # never exceeds the sweep it belongs to
         bytes_launch = part_step_bytes(wl, part_sizes)
         part_ms = ms_local / wl["B"]
         achieved = bytes_launch / (part_ms / 1e3) / 1e9
-        share = grad_ms / max(kern_ms, 1e-12)
         roofline = {"bound": "hbm", "achieved": achieved, "peak": hbm_peak, "unit": "GB/s",
                     "frac": achieved / hbm_peak, "traffic": kernel_traffic(wl_name),
                     "kernel": "part_step (gradient and update)", "kernel_ms": part_ms,
                     "kernel_ms_source": "timed sweeps / B",
-                    "grad_share": share, "update_share": 1.0 - share,
-                    "profiled_grad_kernel_ms": grad_ms, "profiled_update_kernel_ms": upd_ms,
+                    "profiled_part_step_ms": kern_ms,
                     "algorithmic_bytes_per_launch": bytes_launch,
                     "bytes_formula": "8 n_Pi + 4 (I + B) + 8 (I + J) K + 8 J K",
                     "peak_source": f"{peak_src} HBM copy bandwidth"}
@@ -550,9 +547,9 @@ def run_ours(args, wl_name, wl):
                    "parallelism": f"replicas x{world}" if world > 1 else "single GPU"},
         "roofline": roofline,
         # per part-step: the chain kernel and the update (tensor-core path),
-        # or one launch of both (sparse path; four with few entries per row,
-        # counted here as one); per sweep one more (posterior sums and the t
-        # counter)
+        # or one launch of both (sparse path: every workload here has too many
+        # entries per row for the form of four launches); per sweep one more
+        # (posterior sums and the t counter)
         "gpu_launches": args.steps * ((2 if tensor_path(wl) else 1) * wl["B"] + 1),
         "clocks": clocks,
         "rmse_after": rmse,

@@ -96,7 +96,11 @@ typedef struct {
                                *    I*J entries, FP32 gather path);
                                * 1: on, kernel chosen: two-sided (single-pass with
                                *    dense_fp8, and for blocks of at most 128 rows
-                               *    with K <= 128 when V's tiles find no memory);
+                               *    with K <= 128 when V's tiles find no memory).
+                               *    The two-sided kernel holds V as tiles beside
+                               *    the FP32 copy, once or in both orientations:
+                               *    two or three times the single-pass kernel's
+                               *    bytes of V (psgld_estimate_device_bytes);
                                * 2: on, two-sided kernel (K <= 256);
                                * 3: on, single-pass kernel (K <= 128, FP32 V) */
     int32_t dense_v_bf16;     /* 1: the two-sided kernel keeps V in BF16 */
@@ -140,15 +144,15 @@ typedef struct {
                                * not depend on it. */
     int32_t debug_wait_polls; /* for testing the timeout path; 0 (the default): the
                                * normal limit of every bounded device wait (2^24
-                               * polls or about one second of SM clock).  > 0: each
-                               * block of the sparse part-step kernel first makes
-                               * a bulk copy of a row and waits for it with at
-                               * most this many polls, made before it issues the
-                               * copy -- a wait that surely runs out, on purpose:
-                               * the kernel sets the context's error flag, waits
-                               * for the copy with the normal limit and returns
-                               * without a step, and the next synchronising call
-                               * returns
+                               * polls or about one second of SM clock).  > 0: the
+                               * sparse part-step's first wait makes at most this
+                               * many polls, before it issues its copies (with few
+                               * entries per row the row gathers, else a bulk copy
+                               * of one row, made for this in each block) -- a wait
+                               * that surely runs out, on purpose: the kernel sets
+                               * the context's error flag, waits for the copies
+                               * with the normal limit and returns without a step,
+                               * and the next synchronising call returns
                                * PSGLD_ERR_TIMEOUT naming the kernel and the wait.
                                * The part-step's result is then undefined; the
                                * context stays usable (set the factors again). */
@@ -352,10 +356,11 @@ PSGLD_API psgld_status psgld_part_layout(psgld_ctx *ctx, int32_t s, int32_t *row
  * the context's last stream. */
 PSGLD_API psgld_status psgld_profile_read(psgld_ctx *ctx, double *total_ms_host,
                                           int64_t *launches_host);
-/* The same split at the end of the tensor-core chain: *grad_ms_host and
+/* The same split at the end of the gradient launches: *grad_ms_host and
  * *update_ms_host receive the summed durations of the gradient and of the
- * update launches.  On the sparse path gradient and update are one launch,
- * counted as the gradient's. */
+ * update launches.  Sparse part-steps are one launch of both, counted as the
+ * gradient's, except with few entries per row, where they are two launches
+ * (on one stream while profile = 1). */
 PSGLD_API psgld_status psgld_profile_read_split(psgld_ctx *ctx, double *grad_ms_host,
                                                 double *update_ms_host, int64_t *launches_host);
 
@@ -446,7 +451,11 @@ typedef struct {
     double tweedie_p, phi;
     psgld_prior prior;
     psgld_options options;    /* seed, step size, burn_in_sweeps, dense_path
-                               * (1, 2 or 3), dense_v_bf16, ... as for a context */
+                               * (1, 2 or 3), dense_v_bf16, ... as for a context,
+                               * but use_graphs is ignored: the loop launches
+                               * directly (a capture on its thread would make a
+                               * device-wide synchronise of the caller fail while
+                               * it lasts) */
     int32_t sweeps;           /* sweeps to run, > 0 */
     const float *V_dev;       /* I x J, row stride ldv >= J, FP32, device memory */
     int64_t ldv;

@@ -2493,6 +2493,8 @@ psgld_status build_dense_shadows(psgld_ctx *c, cudaStream_t st)
     return PSGLD_OK;
 }
 
+int rc_tile_rows(int64_t max_rows) { return max_rows >= 128 ? 128 : 32 * (int)((max_rows + 31) / 32); }
+
 // Blocks whose columns items cover 256 rows (two accumulators sharing each W
 // tile: a third fewer bytes per MAC); the last blocks' columns items, which
 // end the launch, keep 128 rows so that its CTAs finish together.  The
@@ -2503,8 +2505,6 @@ psgld_status build_dense_shadows(psgld_ctx *c, cudaStream_t st)
 // part's items fill more than one wave of CTAs; short pieces or a single
 // wave favour columns items that form their own mu, all items at once.
 // The option overrides the rule (-1 = the rule).
-int rc_tile_rows(int64_t max_rows) { return max_rows >= 128 ? 128 : 32 * (int)((max_rows + 31) / 32); }
-
 int two_sided_share(int opt, int64_t max_rows, int B, int mt, int nt, int sms)
 {
     if (opt >= 0) return opt;

@@ -4,13 +4,16 @@
 //   W[2]  : I x ldk fp32, row-major, ping-pong pair (ldk = 4*ceil(K/4); the
 //           padding columns are kept at zero so every row is float4-aligned)
 //   Ht[2] : J x ldk fp32, H transposed, same rules
-//   G     : (I + J) x ldk fp32, dense path: the likelihood gradient of the
-//           current part-step (rows 0..I-1 for W, I..I+J-1 for H^T)
+//   G     : (I + J) x ldk fp32, the likelihood gradient of the current
+//           part-step (rows 0..I-1 for W, I..I+J-1 for H^T) on the dense path
+//           and by units; between part-steps read-backs form moments in it
 //   A-side layout (part-major CSR): entries ordered by (part s, row i, col j)
 //           ptrA[s*I + i] .. ptrA[s*I + i + 1] -> idxA (col j), valA (v)
 //   B-side layout (part-major CSC): entries ordered by (part s, col j, row i)
 //           ptrB[s*J + j] .. -> idxB (row i), valB (v)
 //   mid/heavy, per side: per part, the rows with many entries in it
+//   own, unit_sums: contexts that step by units, per side: the entries' own
+//           rows (the A side's in every sparse context), the units' slots
 //   posterior sums: fp64 copies of W, W^2, Ht, Ht^2 (padded like the factors)
 //   dense tensor-core path instead of the two layouts:
 //   Vd    : I x J fp32, row-major (ldv = J)
@@ -377,24 +380,6 @@ __device__ __forceinline__ void wait_prior() { asm volatile("griddepcontrol.wait
 
 // The next kernel's blocks may become resident from here on.
 __device__ __forceinline__ void let_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
-// Philox4x32-10 (Salmon et al., SC'11): ten rounds of two 32x32->64-bit
-// multiplies whose high halves are mixed into the other two words with the
-// round key; the key advances by the Weyl constants between rounds.
-__device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint2 k)
-{
-#pragma unroll
-    for (int r = 0; r < 10; ++r) {
-        if (r > 0) {
-            k.x += 0x9E3779B9u;
-            k.y += 0xBB67AE85u;
-        }
-        const uint32_t lo0 = 0xD2511F53u * c.x, hi0 = __umulhi(0xD2511F53u, c.x);
-        const uint32_t lo1 = 0xCD9E8D57u * c.z, hi1 = __umulhi(0xCD9E8D57u, c.z);
-        c = make_uint4(hi1 ^ c.y ^ k.x, lo1, hi0 ^ c.w ^ k.y, lo0);
-    }
-    return c;
-}
 
 // Uniform on (0, 1): the top 23 bits plus one half, times 2^-23 (exact in
 // fp32).  Then Box-Muller on (u0, u1) and (u2, u3): cos first, then sin.

@@ -1,8 +1,9 @@
 // psgld_step.cu -- one PSGLD iteration (Algorithm 1's loop body), and the
 // update kernels of the dense tensor-core path.
 //
-// On sparse data an iteration is one launch (psgld_rows.cu).  On dense data
-// kept for the tensor cores (dense_path) it is two: the likelihood gradient
+// On sparse data an iteration is one launch (psgld_rows.cu) or, with few
+// entries per row, a gradient and an update launch per factor
+// (psgld_units.cu).  On dense data kept for the tensor cores (dense_path) it is two: the likelihood gradient
 // G of every row of W and H^T (psgld_dense.cu), then the update here, a
 // flat, fully coalesced pass over every (row, float4 group) item of both
 // factors: the row's gradient, Philox4x32-10 normals (counter = group, row,

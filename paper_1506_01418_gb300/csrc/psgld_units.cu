@@ -18,9 +18,9 @@
 // item: the row's gradient (nothing for an empty row), noise, prior, step,
 // mirror; reads X_cur, writes X_next.
 //
-// Sweeps of 3 10^5 x 5000, 10^6 entries, B = 16, at K = 16, 50, 100: 355, 855,
-// 1559 us, with CUDA's logf, sqrtf and sincospif in the normals 404, 984, 1787;
-// one launch of psgld_rows.cu: 470, 1200, 1881.
+// Sweeps of 3 10^5 x 5000, 1.2 10^6 entries, B = 16, at K = 16, 48, 100: 365,
+// 873, 1841 us, with CUDA's logf, sqrtf and sincospif in the normals 395, 963,
+// 1905; one launch of psgld_rows.cu: 532, 1064, 2314.
 #include <algorithm>
 #include <cstring>
 #include <vector>
