@@ -42,16 +42,19 @@
 //
 // What bounds it: instructions and the latency of the gathers.  Of 10^8
 // entries, K = 100, B = 64 (W beyond L2) a part-step's light rows without any
-// entry take 114 us, 92 M warp instructions at 0.66 per cycle and scheduler,
+// entry take 119 us, 100 M warp instructions at 0.70 per cycle and scheduler,
 // most of them Philox and the normals (their rows come into L2 a warp's share
-// at a time: 118 us without).  Against the gradient and the update as two
-// launches per side on two streams (before): 281 instead of 314 us a part-step
-// there; 41.9 instead of 45.8 us with 10^7 entries, K = 50, B = 32 (factors in
-// L2); and one launch instead of four where launches count: a sweep of 256 x
-// 256 dense counts, K = 8, B = 4, and its read-back 31 instead of 48 us.
-// Thresholds measured on the first two, ms a sweep with light up to 16, mid up
-// to 128 and chunks of 512 18.0 and 1.34: 8, 128, 512: 18.3 and 1.43; 32, 128,
-// 512: 18.4 and 1.44; 16, 96, 384: 18.9 and 1.37; 16, 192, 768: 18.2 and 1.38.
+// at a time, 3 % less than without).  Against the gradient and the update as
+// two launches per side on two streams (before): 272 instead of 314 us a
+// part-step there; 41.7 instead of 45.8 us with 10^7 entries, K = 50, B = 32
+// (factors in L2); and one launch instead of four where launches count: a sweep
+// of 256 x 256 dense counts, K = 8, B = 4, and its read-back 32 instead of 48 us.
+// The factors are read by ordinary loads (launch_early); through the read-only
+// path the two took 281 and 41.9 us with a cheaper square root in the normals.
+// Thresholds measured on the first two then, ms a sweep with light up to 16,
+// mid up to 128 and chunks of 512 18.0 and 1.34: 8, 128, 512: 18.3 and 1.43;
+// 32, 128, 512: 18.4 and 1.44; 16, 96, 384: 18.9 and 1.37; 16, 192, 768: 18.2
+// and 1.38.
 #include <algorithm>
 #include <cstring>
 #include <vector>
@@ -561,7 +564,7 @@ RowKernel rows() { return {T, T * NG, rows_kernel<T, NG, U, UM, BF, MINB>}; }
 // Lanes per team and groups per lane for ng float4 groups, entries together
 // (light rows, others), and blocks per SM to hold the registers to.  Warps in
 // flight count most: 64 registers give 32 per SM, which two groups a lane and
-// two entries together fit.  Sweeps of 10^8 entries, K = 100 (and of 3 10^7,
+// two entries together fit but for 40 to 64 bytes of spills.  Sweeps of 10^8 entries, K = 100 (and of 3 10^7,
 // BF16): 16 x 2 with 2 entries 18.0 (13.6) ms, with 4 in 80 registers 18.6
 // (14.3), 32 x 1 19.2 (14.2), 8 x 4 in 114 registers (16 warps) 24.7; of 10^7,
 // K = 50: 8 x 2 with 2 entries 1.34 ms, 16 x 1 with 4 1.37, with 2 1.46.
