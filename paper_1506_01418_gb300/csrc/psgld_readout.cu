@@ -35,12 +35,13 @@ __global__ void moments_kernel(const double *__restrict__ s, const double *__res
 
 constexpr size_t kHalf = 4 << 20;      // staging: two halves, one filled while the other is emptied
 constexpr size_t kSlice = 256 << 10;   // bytes a thread copies at a time
-constexpr size_t kDirect = 1 << 20;    // read-backs up to this go without staging
-// and up to this the sums come over and are divided on the host, which saves
-// four launches.  Moments of 0.4, 0.6, 0.9 MB: 101, 121, 148 us on the host,
-// 125, 129, 135 formed on the device; of 1.3 and 1.8 MB through staging 192 and
-// 229, divided on the host 186 and 235.
-constexpr size_t kHost = 768 << 10;
+// Up to this the sums are copied and divided on the host, one blocking copy at a
+// time.  Moments of 0.05, 0.4, 0.8, 1.3, 1.6 MB, K = 16: 60, 96, 138, 191, 219 us
+// (into new memory 104, 150, 201, 260, 303), through staging -, -, -, 196, 216
+// (-, -, -, 243, 273).  Copied from the device straight to the caller's arrays
+// 0.8 to 1 MB take 140 us, but 890 into new memory; four asynchronous copies and
+// one wait instead of the blocking ones 66, 103, 139.
+constexpr size_t kHost = 1536 << 10;
 // bytes per helping thread: of 1.8 MB with seven 666 us, with none 229; of 8 MB
 // 866, 776 with one, 897 with none; of 40 MB 1509, 3562 with none
 constexpr int64_t kPerHelper = 4 << 20;
@@ -48,7 +49,7 @@ constexpr unsigned kThreads = 8;
 
 // Staging areas of the process, at most kAreas (64 MB), one to a read-back
 // while it lasts, given back with the last context.  A read-back that finds
-// them all taken goes without.
+// them all taken divides on the host.
 constexpr int kAreas = 8;
 std::mutex g_stage_mutex;
 char *g_free[kAreas];
@@ -174,31 +175,24 @@ cudaError_t form(psgld_ctx *c, const Piece &p, cudaStream_t st)
 }
 
 // The same moments, bit for bit, from the sums on the host.
-psgld_status divide_on_host(psgld_ctx *c, double *const (&out)[2][2], cudaStream_t st)
+psgld_status divide_on_host(psgld_ctx *c, double *const (&out)[2][2])
 {
     const int64_t K = c->K, ldk = c->ldk;
     const double n = (double)c->n_samples;
-    std::vector<double> s[2], s2[2];
-    for (int side = 0; side < 2; ++side) {
-        const Sums &S = side == 0 ? c->sW : c->sH;
-        const size_t len = (size_t)((side == 0 ? c->I : c->J) * ldk);
-        for (int var = 0; var < 2; ++var) {
-            if (!out[side][1] && (var || !out[side][0])) continue;
-            std::vector<double> &to = var ? s2[side] : s[side];
-            to.resize(len);
-            PSGLD_CK(c, cudaMemcpyAsync(to.data(), var ? S.s2 : S.s, sizeof(double) * len, cudaMemcpyDeviceToHost, st));
-        }
-    }
-    PSGLD_CK(c, cudaStreamSynchronize(st));
     for (int side = 0; side < 2; ++side) {
         double *const mean = out[side][0], *const var = out[side][1];
-        const int64_t rows = mean || var ? (side == 0 ? c->I : c->J) : 0;
+        if (!mean && !var) continue;
+        const Sums &S = side == 0 ? c->sW : c->sH;
+        const int64_t rows = side == 0 ? c->I : c->J;
+        std::vector<double> s((size_t)(rows * ldk)), s2(var ? s.size() : 0);
+        PSGLD_CK(c, cudaMemcpy(s.data(), S.s, sizeof(double) * s.size(), cudaMemcpyDeviceToHost));
+        if (var) PSGLD_CK(c, cudaMemcpy(s2.data(), S.s2, sizeof(double) * s2.size(), cudaMemcpyDeviceToHost));
         for (int64_t r = 0; r < rows; ++r)
             for (int64_t k = 0; k < K; ++k) {
                 const int64_t at = r * ldk + k;
-                const double m = n > 0 ? s[side][at] / n : 0.0;
+                const double m = n > 0 ? s[at] / n : 0.0;
                 if (mean) mean[r * K + k] = m;
-                if (var) var[r * K + k] = n > 0 ? std::fma(-m, m, s2[side][at] / n) : 0.0;
+                if (var) var[r * K + k] = n > 0 ? std::fma(-m, m, s2[at] / n) : 0.0;
             }
     }
     return PSGLD_OK;
@@ -217,31 +211,26 @@ void use_staging(int by)
 psgld_status read_moments(psgld_ctx *c, double *const (&out)[2][2])
 {
     const size_t row = sizeof(double) * (size_t)c->K;
+    int64_t total = 0;
+    for (int side = 0; side < 2; ++side)
+        for (int var = 0; var < 2; ++var)
+            if (out[side][var]) total += (side == 0 ? c->I : c->J) * (int64_t)row;
+    if (total <= (int64_t)kHost) return divide_on_host(c, out);
+    Staging staging;
+    int readers = 1;
+    char *const area = staging.take(&readers);
+    if (!area) return divide_on_host(c, out);
     const int64_t fit = (int64_t)(sizeof(float) * (size_t)((c->I + c->J) * c->ldk) / row);   // rows G holds
     const int64_t half = std::max<int64_t>(1, std::min<int64_t>(fit, kHalf / row));
     std::vector<Piece> pieces;
-    int64_t total = 0;
     for (int side = 0; side < 2; ++side)
         for (int var = 0; var < 2; ++var) {
             const int64_t rows = side == 0 ? c->I : c->J;
             if (!out[side][var]) continue;
-            total += rows * (int64_t)row;
             for (int64_t r = 0; r < rows; r += half)
                 pieces.push_back({side, var, r, std::min(half, rows - r), out[side][var] + r * c->K});
         }
     cudaStream_t st = c->capture_stream;
-    if (total <= (int64_t)kHost) return divide_on_host(c, out, st);
-    Staging staging;
-    int readers = 1;
-    char *const area = total > (int64_t)kDirect ? staging.take(&readers) : nullptr;
-    if (!area) {
-        for (const Piece &p : pieces) {
-            PSGLD_CK(c, form(c, p, st));
-            PSGLD_CK(c, cudaMemcpyAsync(p.out, c->G, row * (size_t)p.rows, cudaMemcpyDefault, st));
-        }
-        PSGLD_CK(c, cudaStreamSynchronize(st));
-        return PSGLD_OK;
-    }
     cudaEvent_t full[2] = {nullptr, nullptr};
     cudaError_t e = cudaSuccess;
     for (auto &ev : full)
