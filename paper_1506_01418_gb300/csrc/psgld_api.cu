@@ -496,27 +496,32 @@ psgld_status psgld_set_data_coo(psgld_ctx *c, int64_t nnz, const int32_t *i, con
         if (!dev) cudaGetLastError();
         return dev;
     };
-    int32_t *di = nullptr, *dj = nullptr;
-    float *dv = nullptr;
-    psgld_status s = PSGLD_OK;
-    auto stage = [&](auto **copy, auto *&src) {
-        if (s != PSGLD_OK || nnz == 0 || here(src)) return;
-        s = alloc(c, copy, nnz, false, st);
-        if (s != PSGLD_OK) return;
-        const cudaError_t e = cudaMemcpyAsync(*copy, src, sizeof(**copy) * nnz, cudaMemcpyDefault, st);
+    // the others through copies in one allocation: 21 255 shuffled entries from
+    // the host 666 us a load, with three 697
+    const void *src[3] = {i, j, v};
+    const size_t bytes = sizeof(int32_t) * (size_t)nnz, slot = (bytes + 255) & ~size_t(255);
+    int n_copies = 0;
+    for (const void *p : src) n_copies += nnz > 0 && !here(p);
+    unsigned char *copies = nullptr;
+    psgld_status s = n_copies > 0 ? alloc(c, &copies, (int64_t)(slot * n_copies), false, st) : PSGLD_OK;
+    unsigned char *to = copies;
+    for (const void *&p : src) {
+        if (s != PSGLD_OK || nnz == 0 || here(p)) continue;
+        const cudaError_t e = cudaMemcpyAsync(to, p, bytes, cudaMemcpyDefault, st);
         if (e != cudaSuccess) s = cuda_fail(c, e, "copy entries");
-        src = *copy;
-    };
-    stage(&di, i);
-    stage(&dj, j);
-    stage(&dv, v);
+        p = to;
+        to += slot;
+    }
+    i = static_cast<const int32_t *>(src[0]);
+    j = static_cast<const int32_t *>(src[1]);
+    v = static_cast<const float *>(src[2]);
     if (s == PSGLD_OK) s = build_layout(c, nnz, i, j, v, st);
     if (s == PSGLD_OK) s = zero_posterior(c, st);
     if (s == PSGLD_OK) {
         cudaError_t e = cudaStreamSynchronize(st);
         if (e != cudaSuccess) s = cuda_fail(c, e, "sync");
     }
-    dev_free(c, di); dev_free(c, dj); dev_free(c, dv);
+    dev_free(c, copies);
     return s;
 }
 
